@@ -12,6 +12,39 @@
 
 namespace hdcg {
 
+// hi = RN(v), lo = RN(v - hi) of a double whose hi and lo are both normal
+// floats (2^-74 <= |v| < 2^127) or zero, else false; in integer arithmetic: the
+// FP64 pipe does two lanes per clock and SM, so the four FP64 conversions and
+// subtractions per value bound every field conversion (a 16^4 x 16 field went
+// in at 97 us; 50 us with this, the field's traffic at the copy rate is 30 us).
+__device__ __forceinline__ bool split_double(double v, float& hi, float& lo) {
+  const unsigned h = (unsigned)__double2hiint(v), l = (unsigned)__double2loint(v);
+  const unsigned e = (h >> 20) & 0x7ffu;
+  if (e - 949u > 200u) {
+    hi = __uint_as_float(h);
+    lo = 0.f;
+    return ((h << 1) | l) == 0u;
+  }
+  const unsigned top = ((h & 0xfffffu) << 3) | (l >> 29);    // 23 fraction bits
+  const unsigned rem = l & 0x1fffffffu;                      // the 29 below them
+  const unsigned up = (rem > 0x10000000u || (rem == 0x10000000u && (top & 1u))) ? 1u : 0u;
+  hi = __uint_as_float((h & 0x80000000u) | (((e - 896u) << 23 | top) + up));
+  int r = (int)rem - (int)(up << 29);                        // (v - hi) 2^(1075 - e), exact
+  if (h & 0x80000000u) r = -r;
+  lo = __fmul_rn(__int2float_rn(r), __uint_as_float((e - 948u) << 23));   // a power of two
+  return true;
+}
+// the double of a normal float or zero, else false
+__device__ __forceinline__ bool widen_float(float f, double& d) {
+  const unsigned u = __float_as_uint(f), e = (u >> 23) & 0xffu;
+  if (e - 1u > 253u) {
+    d = __hiloint2double((int)u, 0);
+    return (u << 1) == 0u;
+  }
+  d = __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(u << 29));
+  return true;
+}
+
 struct dfl {
   float hi, lo;
   dfl() = default;
@@ -19,10 +52,16 @@ struct dfl {
   __device__ __forceinline__ dfl(int v) : hi((float)v), lo(0.f) {}
   __device__ __forceinline__ dfl(float v) : hi(v), lo(0.f) {}
   __device__ __forceinline__ dfl(double v) {
-    hi = __double2float_rn(v);
-    lo = __double2float_rn(v - (double)hi);
+    if (!split_double(v, hi, lo)) {
+      hi = __double2float_rn(v);
+      lo = __double2float_rn(v - (double)hi);
+    }
   }
-  __device__ __forceinline__ explicit operator double() const { return (double)hi + (double)lo; }
+  __device__ __forceinline__ explicit operator double() const {
+    double h, l;
+    if (widen_float(hi, h) && widen_float(lo, l)) return h + l;
+    return (double)hi + (double)lo;
+  }
 };
 
 // s + e = a + b exactly (TwoSum)
