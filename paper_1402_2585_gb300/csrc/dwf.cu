@@ -178,14 +178,14 @@ static double hop_bytes(const Ctx& c, int pass, int prec, bool extra) {
   return (double)c.n5 * (reals_field * fb + 8.0 * 18.0 * lb / c.Ls);
 }
 
-static void dispatch_hop(int prec, int v, int pass, bool mob, const HopArgs& a, dim3 grid, cudaStream_t st) {
+static void dispatch_hop(int prec, int v, int pass, bool mob, const HopArgs& a, dim3 grid, int threads, cudaStream_t st) {
   switch (prec) {
-    case HDCG_F64: launch_hop_f64(v, pass, mob, a, grid, st); break;
-    case HDCG_F32: launch_hop_f32(v, pass, mob, a, grid, st); break;
-    case HDCG_F16: launch_hop_f16(v, pass, mob, a, grid, st); break;
-    case HDCG_BF16: launch_hop_bf16(v, pass, mob, a, grid, st); break;
-    case HDCG_BF16T: launch_hop_bf16t(v, pass, mob, a, grid, st); break;
-    case HDCG_DF64: launch_hop_df(v, pass, mob, a, grid, st); break;
+    case HDCG_F64: launch_hop_f64(v, pass, mob, a, grid, threads, st); break;
+    case HDCG_F32: launch_hop_f32(v, pass, mob, a, grid, threads, st); break;
+    case HDCG_F16: launch_hop_f16(v, pass, mob, a, grid, threads, st); break;
+    case HDCG_BF16: launch_hop_bf16(v, pass, mob, a, grid, threads, st); break;
+    case HDCG_BF16T: launch_hop_bf16t(v, pass, mob, a, grid, threads, st); break;
+    case HDCG_DF64: launch_hop_df(v, pass, mob, a, grid, threads, st); break;
     default: throw Error{HDCG_ERR_ARG, "unknown precision code"};
   }
 }
@@ -193,7 +193,7 @@ static void dispatch_hop(int prec, int v, int pass, bool mob, const HopArgs& a, 
 // Hop autotuner: the first launch of a (precision, pass, fused-CG) combination
 // times every register-budget variant on scratch fields (never on the
 // caller's data, so in-place CG updates are not repeated) and keeps the fastest.
-static int hop_variant(Ctx& c, int prec, int pass, bool mob, const HopArgs& a, dim3 grid) {
+static int hop_variant(Ctx& c, int prec, int pass, bool mob, const HopArgs& a, dim3 grid, int threads) {
   const int key = ((prec * 4 + pass) * 2 + (a.cg_r ? 1 : 0)) * 2 + (a.do_red ? 1 : 0);
   if (c.hop_force >= 0) {
     // a forced variant (hdcg_set_hop_variant); the packed variants exist for
@@ -237,9 +237,9 @@ static int hop_variant(Ctx& c, int prec, int pass, bool mob, const HopArgs& a, d
   // run only when forced
   const int nv = 4;
   for (int v = 0; v < nv; ++v) {
-    dispatch_hop(prec, v, pass, mob, t, grid, c.stream);  // warm-up
+    dispatch_hop(prec, v, pass, mob, t, grid, threads, c.stream);  // warm-up
     HDCG_CUDA(cudaEventRecord(e0, c.stream));
-    for (int r = 0; r < 3; ++r) dispatch_hop(prec, v, pass, mob, t, grid, c.stream);
+    for (int r = 0; r < 3; ++r) dispatch_hop(prec, v, pass, mob, t, grid, threads, c.stream);
     HDCG_CUDA(cudaEventRecord(e1, c.stream));
     HDCG_CUDA(cudaEventSynchronize(e1));
     float ms = 0.f;
@@ -258,6 +258,14 @@ static int hop_variant(Ctx& c, int prec, int pass, bool mob, const HopArgs& a, d
   // 32^3 x 64 x 16 FP64 field)
   for (int i = 20; i < 24; ++i) c.scratch_f[prec][i].release();
   return best;
+}
+
+// Threads per CTA.  FP64 and double-float kernels are built for 64.  The others
+// run 256, and 64 while that leaves SMs idle (152 SMs; an 8^4 x 8 field is 64
+// CTAs of 256 threads).
+static int hop_threads(const Ctx& c, int prec, int nrhs) {
+  if (prec == HDCG_F64 || prec == HDCG_DF64) return 64;
+  return c.n5 * (size_t)nrhs < (size_t)152 * 256 * 2 ? 64 : 256;
 }
 
 void launch_hop(Ctx& c, int pass, int prec, const uint4* in, const uint4* in2, uint4* out,
@@ -283,15 +291,19 @@ void launch_hop(Ctx& c, int pass, int prec, const uint4* in, const uint4* in2, u
   for (int j = 0; j < 6; ++j) a.rpow[j] = c.co.rpow[j];
   a.sD = epi.sD;
   a.lam = epi.lam;
-  a.fb = (float)a.b;
-  a.fc = (float)a.c;
-  a.falpha = (float)a.alpha;
-  a.fbeta = (float)a.beta;
-  a.fmass = (float)a.mass;
-  a.fminv_norm = (float)a.minv_norm;
-  for (int j = 0; j < 6; ++j) a.frpow[j] = (float)a.rpow[j];
-  a.fsD = (float)a.sD;
-  a.flam = (float)a.lam;
+  const auto split = [](double d, float& f, float& l) {
+    f = (float)d;
+    l = (float)(d - (double)f);
+  };
+  split(a.b, a.fb, a.lb);
+  split(a.c, a.fc, a.lc);
+  split(a.alpha, a.falpha, a.lalpha);
+  split(a.beta, a.fbeta, a.lbeta);
+  split(a.mass, a.fmass, a.lmass);
+  split(a.minv_norm, a.fminv_norm, a.lminv_norm);
+  for (int j = 0; j < 6; ++j) split(a.rpow[j], a.frpow[j], a.lrpow[j]);
+  split(a.sD, a.fsD, a.lsD);
+  split(a.lam, a.flam, a.llam);
   a.cg_x = epi.cg_x;
   a.cg_r = epi.cg_r;
   a.cg_p = epi.cg_p;
@@ -301,7 +313,8 @@ void launch_hop(Ctx& c, int pass, int prec, const uint4* in, const uint4* in2, u
   a.al_lam = epi.al_lam;
   a.fstride = epi.nrhs > 1 ? epi.fstride : 0;
   a.al_mask = epi.mask;
-  const unsigned grid = (unsigned)((c.n5 + 255) / 256);
+  const int threads = hop_threads(c, prec, epi.nrhs);
+  const unsigned grid = (unsigned)((c.n5 + threads - 1) / threads);
   HDCG_REQUIRE(epi.nrhs >= 1 && epi.nrhs <= RMAX, HDCG_ERR_ARG, "1 <= right-hand sides <= 16");
   a.do_red = red_result != nullptr;
   if (a.do_red) {
@@ -314,14 +327,14 @@ void launch_hop(Ctx& c, int pass, int prec, const uint4* in, const uint4* in2, u
   }
   const bool mob = c.co.c != 0.0;
   const dim3 grid2(grid, (unsigned)epi.nrhs);
-  const int v = hop_variant(c, prec, pass, mob, a, grid2);
+  const int v = hop_variant(c, prec, pass, mob, a, grid2, threads);
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
   if (c.prof.on) {
     HDCG_CUDA(cudaEventCreate(&ev0));
     HDCG_CUDA(cudaEventCreate(&ev1));
     HDCG_CUDA(cudaEventRecord(ev0, c.stream));
   }
-  dispatch_hop(prec, v, pass, mob, a, grid2, c.stream);
+  dispatch_hop(prec, v, pass, mob, a, grid2, threads, c.stream);
   HDCG_CUDA(cudaGetLastError());
   ++c.launches;
   if (c.prof.on) {

@@ -22,9 +22,11 @@ struct HopArgs {
   int Ls, lslog2;
   double b, c, alpha, beta, mass, minv_norm, rpow[6];
   double sD, lam;
-  // the same coefficients rounded to float on the host: the FP32/16-bit passes
-  // read these, so no thread converts from double (GB300's FP64 pipe is narrow)
+  // the same coefficients rounded to float on the host (f*), and what that
+  // rounding left (l*): the FP32/16-bit and double-float passes read these, so
+  // no thread converts from double (GB300's FP64 pipe is narrow)
   float fb, fc, falpha, fbeta, fmass, fminv_norm, frpow[6], fsD, flam;
+  float lb, lc, lalpha, lbeta, lmass, lminv_norm, lrpow[6], lsD, llam;
   Reduction red;
   int do_red;
   // fused CG step in pass D (cg_r != null): w = out is not stored; instead
@@ -44,9 +46,11 @@ struct HopArgs {
 };
 
 // coefficient in the arithmetic type R: the host-rounded float for FP32
-// arithmetic, the double otherwise (FP64 and double-float passes)
-template <typename R> __device__ __forceinline__ R sc(double d, float) { return R(d); }
-template <> __device__ __forceinline__ float sc<float>(double, float f) { return f; }
+// arithmetic, the double for FP64, both parts for double-float
+template <typename R> __device__ __forceinline__ R sc(double d, float f, float l);
+template <> __device__ __forceinline__ double sc<double>(double d, float, float) { return d; }
+template <> __device__ __forceinline__ float sc<float>(double, float f, float) { return f; }
+template <> __device__ __forceinline__ dfl sc<dfl>(double, float f, float l) { return dfl(f, l); }
 
 // ------------------------------------------------------------------------------
 // link loads: 9 complex of one link into 18 reals.  Links are stored padded to
@@ -138,29 +142,29 @@ __device__ __forceinline__ void apply_lin(R* v, R a, R b, int s, int Ls, R m) {
   const int sp = DAG ? up_src : dn_src, sm = DAG ? dn_src : up_src;
   const R bp = b * (DAG ? up_f : dn_f), bm = b * (DAG ? dn_f : up_f);
 #pragma unroll
-  for (int i = 0; i < 12; ++i) v[i] = a * v[i] + bp * shfl_any(v[i], sp, Ls);
+  for (int i = 0; i < 12; ++i) v[i] = madd2(a, v[i], bp, shfl_any(v[i], sp, Ls));
 #pragma unroll
-  for (int i = 12; i < 24; ++i) v[i] = a * v[i] + bm * shfl_any(v[i], sm, Ls);
+  for (int i = 12; i < 24; ++i) v[i] = madd2(a, v[i], bm, shfl_any(v[i], sm, Ls));
 }
 
 // v <- M_ee^-1 v (DAG: M_ee^-dag) by doubling: A_{j+1} = A_j + r^{2^j} P^{2^j} A_j
 template <typename R, bool DAG>
 __device__ __forceinline__ void apply_minv(R* v, int s, const HopArgs& a) {
-  const R m = sc<R>(a.mass, a.fmass);
+  const R m = sc<R>(a.mass, a.fmass, a.lmass);
   const int Ls = a.Ls;
   for (int j = 0; j < a.lslog2; ++j) {
     const int d = 1 << j;
     const int up_src = (s + d) & (Ls - 1), dn_src = (s - d) & (Ls - 1);
     const R up_f = (s + d >= Ls) ? -m : R(1), dn_f = (s < d) ? -m : R(1);
     const int sp = DAG ? up_src : dn_src, sm = DAG ? dn_src : up_src;
-    const R rp = sc<R>(a.rpow[j], a.frpow[j]);
+    const R rp = sc<R>(a.rpow[j], a.frpow[j], a.lrpow[j]);
     const R cp = rp * (DAG ? up_f : dn_f), cm = rp * (DAG ? dn_f : up_f);
 #pragma unroll
-    for (int i = 0; i < 12; ++i) v[i] += cp * shfl_any(v[i], sp, Ls);
+    for (int i = 0; i < 12; ++i) v[i] = madd(cp, shfl_any(v[i], sp, Ls), v[i]);
 #pragma unroll
-    for (int i = 12; i < 24; ++i) v[i] += cm * shfl_any(v[i], sm, Ls);
+    for (int i = 12; i < 24; ++i) v[i] = madd(cm, shfl_any(v[i], sm, Ls), v[i]);
   }
-  const R nrm = sc<R>(a.minv_norm, a.fminv_norm);
+  const R nrm = sc<R>(a.minv_norm, a.fminv_norm, a.lminv_norm);
 #pragma unroll
   for (int i = 0; i < 24; ++i) v[i] *= nrm;
 }
@@ -242,6 +246,77 @@ __device__ __forceinline__ void su3_mul(const R* U, const R* h, R* uh) {
     }
 }
 
+// FP64: one chain of fused multiply-adds per real (6 instructions).  The
+// expression above compiles to 9: the compiler may not reassociate, so each
+// `ur hr - ui hi` is a product and a multiply-add of its own, and the FP64 pipe
+// (two lanes per clock and SM) bounds these passes.  Mpc and Mpc^dag on 8^4 x 8:
+// 389 -> 298 us, with 64-thread CTAs (hop_bound) 168 us.
+__device__ __forceinline__ void su3_mul(const double* U, const double* h, double* uh) {
+#pragma unroll
+  for (int sp = 0; sp < 2; ++sp)
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      double re = 0, im = 0;
+#pragma unroll
+      for (int b = 0; b < 3; ++b) {
+        const double ur = U[(a * 3 + b) * 2], ui = U[(a * 3 + b) * 2 + 1];
+        const double hr = h[(sp * 3 + b) * 2], hi = h[(sp * 3 + b) * 2 + 1];
+        re = b ? fma(ur, hr, re) : ur * hr;
+        im = b ? fma(ur, hi, im) : ur * hi;
+        re = fma(-ui, hi, re);
+        im = fma(ui, hr, im);
+      }
+      uh[(sp * 3 + a) * 2] = re;
+      uh[(sp * 3 + a) * 2 + 1] = im;
+    }
+}
+// double-float: three compensated pairs of products per real, 76 operations
+// against 108 (H on 16^4 x 16: 2.67 -> 2.02 ms together with the 64-thread CTAs
+// below and the split coefficients; error against 64 bits 4.5e-15 both)
+__device__ __forceinline__ void su3_mul(const dfl* U, const dfl* h, dfl* uh) {
+#pragma unroll
+  for (int sp = 0; sp < 2; ++sp)
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      dfl re[3], im[3];
+#pragma unroll
+      for (int b = 0; b < 3; ++b) {
+        const dfl ur = U[(a * 3 + b) * 2], ui = U[(a * 3 + b) * 2 + 1];
+        const dfl hr = h[(sp * 3 + b) * 2], hi = h[(sp * 3 + b) * 2 + 1];
+        re[b] = dot2(ur, hr, -ui, hi);
+        im[b] = dot2(ur, hi, ui, hr);
+      }
+      uh[(sp * 3 + a) * 2] = sum3(re[0], re[1], re[2]);
+      uh[(sp * 3 + a) * 2 + 1] = sum3(im[0], im[1], im[2]);
+    }
+}
+
+// acc += (uf + ub, -SF B_mu (uf - ub)): both hops along mu at once, so that each
+// accumulator takes four summands, not eight
+template <int MU, int SF>
+__device__ __forceinline__ void reconstruct_pair(const dfl* uf, const dfl* ub, dfl* acc) {
+#pragma unroll
+  for (int sp = 0; sp < 2; ++sp)
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const int k = (sp * 3 + c) * 2;
+      acc[k] += lazy_add(uf[k], ub[k]);
+      acc[k + 1] += lazy_add(uf[k + 1], ub[k + 1]);
+      // lower spin sp takes -SF B_mu of the upper spin j: B_x, B_y swap the spins
+      const int j = MU < 2 ? 1 - sp : sp;
+      const int q = (j * 3 + c) * 2;
+      const dfl dr = lazy_add(uf[q], -ub[q]), di = lazy_add(uf[q + 1], -ub[q + 1]);
+      dfl br, bi;   // B_mu d
+      if (MU == 0) { br = -di; bi = dr; }
+      else if (MU == 1) { br = sp == 0 ? dr : -dr; bi = sp == 0 ? di : -di; }
+      else if (MU == 2) { br = sp == 0 ? -di : di; bi = sp == 0 ? dr : -dr; }
+      else { br = dr; bi = di; }
+      const int l = ((2 + sp) * 3 + c) * 2;
+      acc[l] += SF > 0 ? -br : br;
+      acc[l + 1] += SF > 0 ? -bi : bi;
+    }
+}
+
 template <typename St> struct LinkOf;
 template <> struct LinkOf<f64_t> { using T = double2; };
 template <> struct LinkOf<df_t> { using T = float4; };
@@ -258,41 +333,38 @@ __device__ __forceinline__ void hop_pair(const HopArgs& a, const uint4* in, cons
                                          R* acc) {
   constexpr int LG = LinkGran<LT>::g;
   if constexpr (std::is_same<R, dfl>::value) {
-    // double-float: compute-bound, so one neighbour at a time keeps registers low
+    // double-float: bound by arithmetic, so one neighbour at a time keeps registers low
+    R uh[2][12];
 #pragma unroll
     for (int side = 0; side < 2; ++side) {
       R ps[24];
       load_spinor<St, R>(in, (size_t)nbv[MU + 4 * side] * a.Ls + s, a.n5, ps);
-      if (KIN) apply_lin<R, false>(ps, sc<R>(a.b, a.fb), sc<R>(a.c, a.fc), s, a.Ls, sc<R>(a.mass, a.fmass));
-      R h[12], uh[12], U[18];
+      if (KIN)
+        apply_lin<R, false>(ps, sc<R>(a.b, a.fb, a.lb), sc<R>(a.c, a.fc, a.lc), s, a.Ls, sc<R>(a.mass, a.fmass, a.lmass));
+      R h[12], U[18];
       load_link((const LT*)nullptr, lk + (MU + 4 * side) * LG, U);
-      if (side == 0) {
-        project<MU, SF>(ps, h);
-        su3_mul<R>(U, h, uh);
-        reconstruct_add<MU, SF>(uh, acc);
-      } else {
-        project<MU, -SF>(ps, h);
-        su3_mul<R>(U, h, uh);
-        reconstruct_add<MU, -SF>(uh, acc);
-      }
+      if (side == 0) project<MU, SF>(ps, h);
+      else project<MU, -SF>(ps, h);
+      su3_mul(U, h, uh[side]);
     }
+    reconstruct_pair<MU, SF>(uh[0], uh[1], acc);
   } else {
     R pf[24], pb[24];
     load_spinor<St, R>(in, (size_t)nbv[MU] * a.Ls + s, a.n5, pf);
     load_spinor<St, R>(in, (size_t)nbv[MU + 4] * a.Ls + s, a.n5, pb);
     if (KIN) {
-      const R m = sc<R>(a.mass, a.fmass), kb = sc<R>(a.b, a.fb), kc = sc<R>(a.c, a.fc);
+      const R m = sc<R>(a.mass, a.fmass, a.lmass), kb = sc<R>(a.b, a.fb, a.lb), kc = sc<R>(a.c, a.fc, a.lc);
       apply_lin<R, false>(pf, kb, kc, s, a.Ls, m);
       apply_lin<R, false>(pb, kb, kc, s, a.Ls, m);
     }
     R h[12], uh[12], U[18];
     project<MU, SF>(pf, h);
     load_link((const LT*)nullptr, lk + MU * LG, U);
-    su3_mul<R>(U, h, uh);
+    su3_mul(U, h, uh);
     reconstruct_add<MU, SF>(uh, acc);
     project<MU, -SF>(pb, h);
     load_link((const LT*)nullptr, lk + (MU + 4) * LG, U);
-    su3_mul<R>(U, h, uh);
+    su3_mul(U, h, uh);
     reconstruct_add<MU, -SF>(uh, acc);
   }
 }
@@ -311,16 +383,16 @@ __device__ __forceinline__ void hop_raw(const HopArgs& a, const uint4 (&raw)[8][
 #pragma unroll
       for (int i = 0; i < 8; ++i) ps[c * 8 + i] = (R)t[i];
     }
-    if (KIN) apply_lin<R, false>(ps, sc<R>(a.b, a.fb), sc<R>(a.c, a.fc), s, a.Ls, sc<R>(a.mass, a.fmass));
+    if (KIN) apply_lin<R, false>(ps, sc<R>(a.b, a.fb, a.lb), sc<R>(a.c, a.fc, a.lc), s, a.Ls, sc<R>(a.mass, a.fmass, a.lmass));
     R h[12], uh[12], U[18];
     load_link((const LT*)nullptr, lk + (MU + 4 * side) * LG, U);
     if (side == 0) {
       project<MU, SF>(ps, h);
-      su3_mul<R>(U, h, uh);
+      su3_mul(U, h, uh);
       reconstruct_add<MU, SF>(uh, acc);
     } else {
       project<MU, -SF>(ps, h);
-      su3_mul<R>(U, h, uh);
+      su3_mul(U, h, uh);
       reconstruct_add<MU, -SF>(uh, acc);
     }
   }
@@ -379,8 +451,16 @@ template <bool DF> struct HopCompute<df_t, DF> { using type = dfl; };
 // PF (16-bit storage only): the raw 16-byte granules of all eight neighbour
 // spinors are loaded before any is used (24 loads in flight per thread).
 // DF (FP64 storage only): double-float arithmetic instead of FP64 units.
+// FP64 and double-float storage: CTAs of 64 threads, so that the register file
+// is filled in steps of two warps (170 registers: 12 warps per SM, where CTAs
+// of 256 threads leave 8) and small lattices reach every SM; MINB 3 then asks
+// for six of them (168 registers) instead of spilling at 80.
+template <typename St> constexpr int hop_bound() { return Store<St>::chunks == 12 ? 64 : 256; }
+template <typename St, int MINB> constexpr int hop_ctas() {
+  return Store<St>::chunks != 12 ? MINB : MINB == 3 ? 6 : 4 * MINB;
+}
 template <typename St, int PASS, bool MOB, int MINB, bool PF = false, bool DF = false>
-__global__ void __launch_bounds__(256, MINB) hop_kernel(const HopArgs a) {
+__global__ void __launch_bounds__(hop_bound<St>(), hop_ctas<St, MINB>()) hop_kernel(const HopArgs a) {
   using R = typename HopCompute<St, DF>::type;
   using LT = typename LinkOf<St>::T;
   constexpr bool DAG = (PASS == PASS_C || PASS == PASS_D);
@@ -391,8 +471,8 @@ __global__ void __launch_bounds__(256, MINB) hop_kernel(const HopArgs a) {
   const int s = threadIdx.x & (a.Ls - 1);
   const size_t x4 = active ? (gtid >> a.lslog2) : 0;
   const size_t site5 = x4 * a.Ls + s;
-  const R m = sc<R>(a.mass, a.fmass);
-  const R kb = sc<R>(a.b, a.fb), kc = sc<R>(a.c, a.fc);
+  const R m = sc<R>(a.mass, a.fmass, a.lmass);
+  const R kb = sc<R>(a.b, a.fb, a.lb), kc = sc<R>(a.c, a.fc, a.lc);
 
   R acc[24];
 #pragma unroll
@@ -452,17 +532,17 @@ __global__ void __launch_bounds__(256, MINB) hop_kernel(const HopArgs a) {
     }
     R self[24];
     load_spinor<St, R>(a.in2 + roff, site5, a.n5, self);
-    apply_lin<R, DAG>(self, sc<R>(a.alpha, a.falpha), sc<R>(a.beta, a.fbeta), s, a.Ls, m);
+    apply_lin<R, DAG>(self, sc<R>(a.alpha, a.falpha, a.lalpha), sc<R>(a.beta, a.fbeta, a.lbeta), s, a.Ls, m);
 #pragma unroll
     for (int i = 0; i < 24; ++i) acc[i] = self[i] - R(0.25) * acc[i];
     if (PASS == PASS_D) {
-      const R sD = sc<R>(a.sD, a.fsD);
+      const R sD = sc<R>(a.sD, a.fsD, a.lsD);
 #pragma unroll
       for (int i = 0; i < 24; ++i) acc[i] *= sD;
       if (a.extra) {
         R ex[24];
         load_spinor<St, R>(a.extra + roff, site5, a.n5, ex);
-        const R lam = sc<R>(a.lam, a.flam);
+        const R lam = sc<R>(a.lam, a.flam, a.llam);
 #pragma unroll
         for (int i = 0; i < 24; ++i) acc[i] += lam * ex[i];
       }
@@ -471,16 +551,17 @@ __global__ void __launch_bounds__(256, MINB) hop_kernel(const HopArgs a) {
   if (PASS == PASS_D && a.cg_r) {
     // alpha of the fused CG step: one FP64 division per CTA, shared
     __shared__ double s_alpha;
-    __shared__ float s_alphaf;
+    __shared__ float s_alphaf, s_alphal;
     if (threadIdx.x == 0) {
       double den = a.al_den0[rhs];
       if (a.al_den1) den += a.al_lam * a.al_den1[rhs];
       const bool live = a.al_mask == nullptr || a.al_mask[rhs] != 0;
       s_alpha = (den != 0.0 && live) ? a.al_num[rhs] / den : 0.0;
       s_alphaf = (float)s_alpha;
+      s_alphal = (float)(s_alpha - (double)s_alphaf);
     }
     __syncthreads();
-    const R alpha = sc<R>(s_alpha, s_alphaf);
+    const R alpha = sc<R>(s_alpha, s_alphaf, s_alphal);
     if (active) {
       R rv[24], xv[24], pv[24];
       load_spinor<St, R>(a.cg_r + roff, site5, a.n5, rv);
@@ -516,18 +597,18 @@ template <typename St> constexpr int hop_variants() { return Store<St>::chunks =
 
 // launch variant v of one pass for storage St
 template <typename St>
-void launch_hop_variant(int v, int pass, bool mob, const HopArgs& a, dim3 grid, cudaStream_t st) {
+void launch_hop_variant(int v, int pass, bool mob, const HopArgs& a, dim3 grid, int threads, cudaStream_t st) {
   if constexpr (Store<St>::chunks != 12) {
     if (v >= 4) {
       const bool stage = a.Ls >= 8;
 #define HDCG_HOP_PK(P, M)                                                                       \
       if (pass == P) {                                                                         \
         if (stage) {                                                                           \
-          if (mob) pk::hop_packed_kernel<St, P, true, M, true><<<grid, 256, 0, st>>>(a);       \
-          else pk::hop_packed_kernel<St, P, false, M, true><<<grid, 256, 0, st>>>(a);          \
+          if (mob) pk::hop_packed_kernel<St, P, true, M, true><<<grid, threads, 0, st>>>(a);       \
+          else pk::hop_packed_kernel<St, P, false, M, true><<<grid, threads, 0, st>>>(a);          \
         } else {                                                                               \
-          if (mob) pk::hop_packed_kernel<St, P, true, M, false><<<grid, 256, 0, st>>>(a);      \
-          else pk::hop_packed_kernel<St, P, false, M, false><<<grid, 256, 0, st>>>(a);         \
+          if (mob) pk::hop_packed_kernel<St, P, true, M, false><<<grid, threads, 0, st>>>(a);      \
+          else pk::hop_packed_kernel<St, P, false, M, false><<<grid, threads, 0, st>>>(a);         \
         }                                                                                      \
         return;                                                                                \
       }
@@ -542,8 +623,8 @@ void launch_hop_variant(int v, int pass, bool mob, const HopArgs& a, dim3 grid, 
   }
 #define HDCG_HOP_CASE(P, M)                                                      \
   if (pass == P && v == M - 1) {                                                 \
-    if (mob) hop_kernel<St, P, true, M><<<grid, 256, 0, st>>>(a);               \
-    else hop_kernel<St, P, false, M><<<grid, 256, 0, st>>>(a);                  \
+    if (mob) hop_kernel<St, P, true, M><<<grid, threads, 0, st>>>(a);               \
+    else hop_kernel<St, P, false, M><<<grid, threads, 0, st>>>(a);                  \
     return;                                                                      \
   }
   HDCG_HOP_CASE(PASS_A, 1) HDCG_HOP_CASE(PASS_A, 2) HDCG_HOP_CASE(PASS_A, 3)
@@ -556,8 +637,8 @@ void launch_hop_variant(int v, int pass, bool mob, const HopArgs& a, dim3 grid, 
     constexpr bool DF = Store<St>::chunks == 12;
 #define HDCG_HOP_PF(P)                                                           \
     if (pass == P) {                                                             \
-      if (mob) hop_kernel<St, P, true, 1, PF, DF><<<grid, 256, 0, st>>>(a);     \
-      else hop_kernel<St, P, false, 1, PF, DF><<<grid, 256, 0, st>>>(a);        \
+      if (mob) hop_kernel<St, P, true, 1, PF, DF><<<grid, threads, 0, st>>>(a);     \
+      else hop_kernel<St, P, false, 1, PF, DF><<<grid, threads, 0, st>>>(a);        \
       return;                                                                    \
     }
     HDCG_HOP_PF(PASS_A) HDCG_HOP_PF(PASS_B) HDCG_HOP_PF(PASS_C) HDCG_HOP_PF(PASS_D)
@@ -566,11 +647,11 @@ void launch_hop_variant(int v, int pass, bool mob, const HopArgs& a, dim3 grid, 
 }
 
 // explicit instantiations live in dwf_<prec>.cu
-void launch_hop_f64(int v, int pass, bool mob, const HopArgs& a, dim3 grid, cudaStream_t st);
-void launch_hop_f32(int v, int pass, bool mob, const HopArgs& a, dim3 grid, cudaStream_t st);
-void launch_hop_f16(int v, int pass, bool mob, const HopArgs& a, dim3 grid, cudaStream_t st);
-void launch_hop_bf16(int v, int pass, bool mob, const HopArgs& a, dim3 grid, cudaStream_t st);
-void launch_hop_bf16t(int v, int pass, bool mob, const HopArgs& a, dim3 grid, cudaStream_t st);
-void launch_hop_df(int v, int pass, bool mob, const HopArgs& a, dim3 grid, cudaStream_t st);
+void launch_hop_f64(int v, int pass, bool mob, const HopArgs& a, dim3 grid, int threads, cudaStream_t st);
+void launch_hop_f32(int v, int pass, bool mob, const HopArgs& a, dim3 grid, int threads, cudaStream_t st);
+void launch_hop_f16(int v, int pass, bool mob, const HopArgs& a, dim3 grid, int threads, cudaStream_t st);
+void launch_hop_bf16(int v, int pass, bool mob, const HopArgs& a, dim3 grid, int threads, cudaStream_t st);
+void launch_hop_bf16t(int v, int pass, bool mob, const HopArgs& a, dim3 grid, int threads, cudaStream_t st);
+void launch_hop_df(int v, int pass, bool mob, const HopArgs& a, dim3 grid, int threads, cudaStream_t st);
 
 }  // namespace hdcg

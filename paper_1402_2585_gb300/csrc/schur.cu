@@ -13,8 +13,10 @@ namespace hdcg {
 
 namespace {
 
+constexpr int SCHUR_THREADS = 64;   // FP64 passes, as hop_kernel's (hop_bound)
+
 // out = K M_ee^-1 in (s-local, either parity)
-__global__ void k_kminv(const HopArgs a) {
+__global__ void __launch_bounds__(SCHUR_THREADS, 6) k_kminv(const HopArgs a) {
   const size_t gtid = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   const bool active = gtid < a.n5;
   const size_t site5 = active ? gtid : 0;
@@ -29,7 +31,7 @@ __global__ void k_kminv(const HopArgs a) {
 // acc = Dh (K^KIN in) at the output parity; EPI 0: out = in2 + acc / 2,
 // EPI 1: out = M_ee^-1 (in2 + acc / 2)
 template <bool KIN, int EPI>
-__global__ void k_hop_half(const HopArgs a) {
+__global__ void __launch_bounds__(SCHUR_THREADS, 6) k_hop_half(const HopArgs a) {
   const size_t gtid = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   const bool active = gtid < a.n5;
   const int s = threadIdx.x & (a.Ls - 1);
@@ -82,16 +84,16 @@ void prep_source(Ctx& c, const void* eta_e, const void* eta_o, void* b) {
   uint4* t = c.scratch(HDCG_F64, 4);
   canon_to_internal(c, eta_e, HDCG_F64, e, HDCG_F64);
   canon_to_internal(c, eta_o, HDCG_F64, o, HDCG_F64);
-  const unsigned g = (unsigned)((c.n5 + 255) / 256);
+  const unsigned g = (unsigned)((c.n5 + SCHUR_THREADS - 1) / SCHUR_THREADS);
   HopArgs a = args(c, 0);
   a.in = e;
   a.out = t;
-  k_kminv<<<g, 256, 0, c.stream>>>(a);             // t_e = K M_ee^-1 eta_e
+  k_kminv<<<g, SCHUR_THREADS, 0, c.stream>>>(a);             // t_e = K M_ee^-1 eta_e
   a = args(c, 1);
   a.in = t;
   a.in2 = o;
   a.out = e;
-  k_hop_half<false, 0><<<g, 256, 0, c.stream>>>(a);  // eta_o' = eta_o + Dh_oe t_e / 2
+  k_hop_half<false, 0><<<g, SCHUR_THREADS, 0, c.stream>>>(a);  // eta_o' = eta_o + Dh_oe t_e / 2
   HDCG_CUDA(cudaGetLastError());
   c.launches += 2;
   apply_mpc(c, HDCG_F64, e, t, 1, nullptr);         // b = Mpc^dag eta_o'
@@ -106,12 +108,12 @@ void reconstruct(Ctx& c, const void* eta_e, const void* psi_o, void* psi_e) {
   uint4* t = c.scratch(HDCG_F64, 4);
   canon_to_internal(c, eta_e, HDCG_F64, e, HDCG_F64);
   canon_to_internal(c, psi_o, HDCG_F64, o, HDCG_F64);
-  const unsigned g = (unsigned)((c.n5 + 255) / 256);
+  const unsigned g = (unsigned)((c.n5 + SCHUR_THREADS - 1) / SCHUR_THREADS);
   HopArgs a = args(c, 0);
   a.in = o;
   a.in2 = e;
   a.out = t;
-  k_hop_half<true, 1><<<g, 256, 0, c.stream>>>(a);
+  k_hop_half<true, 1><<<g, SCHUR_THREADS, 0, c.stream>>>(a);
   HDCG_CUDA(cudaGetLastError());
   ++c.launches;
   internal_to_canon(c, t, HDCG_F64, psi_e, HDCG_F64);
