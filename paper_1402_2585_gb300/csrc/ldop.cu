@@ -454,7 +454,8 @@ __global__ void k_ad1_p(float2* p, const float2* __restrict__ y, size_t ne, int 
     for (int q = 0; q < RMAX; ++q) {
       if (q < R) {
         const size_t o = t * R + q;
-        float2 pv = p[o];
+        // first: p is work memory nobody wrote yet (0 x NaN would survive beta = 0)
+        float2 pv = first ? make_float2(0.f, 0.f) : p[o];
         if (!ctl->done[q]) {
           float beta = 0.f;
           if (!first) {
@@ -464,8 +465,8 @@ __global__ void k_ad1_p(float2* p, const float2* __restrict__ y, size_t ne, int 
           const float2 yv = y[o];
           pv.x = yv.x + beta * pv.x;
           pv.y = yv.y + beta * pv.y;
-          p[o] = pv;
         }
+        if (first || !ctl->done[q]) p[o] = pv;
         m[q] = fmaxf(fabsf(pv.x), fabsf(pv.y));
       }
     }
