@@ -28,57 +28,135 @@ namespace {
 
 unsigned nblk(size_t n) { return (unsigned)((n + 255) / 256); }
 
-// y[a][j][r] = sum_q sum_k A9[a][q][k][j] x[nb9[a][q]][k][r] + shift x[a][j][r],
-// one warp per coarse site: lane l owns the outputs
-// o = o0 + l + 32 u (u < U) of the current chunk, j = o / R, r = o % R.  Each
-// row of a kept block (fixed q and k) is read coalesced across j, x[nb][k][r]
-// is a broadcast within the warp, and no shared memory or barrier is needed.
-template <int U>
-__global__ void __launch_bounds__(256) k_qtrunc_apply_w(const float2* __restrict__ A9, const int* __restrict__ nb9,
-                                                        int nq, int n, const float2* __restrict__ x, int R,
-                                                        float shift, float2* y, const int* skip, size_t Vc) {
-  if (skip && *skip) return;
-  const size_t a = (size_t)blockIdx.x * 8 + (threadIdx.x >> 5);
-  if (a >= Vc) return;
-  const int lane = threadIdx.x & 31;
-  const int nout = n * R;
-  for (int o0 = 0; o0 < nout; o0 += 32 * U) {
-    float ar[U], ai[U];
-    int jo[U], ro[U];
-    bool live[U];
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int o = o0 + lane + 32 * u;
-      live[u] = o < nout;
-      jo[u] = live[u] ? o / R : 0;
-      ro[u] = live[u] ? o % R : 0;
-      ar[u] = 0.f;
-      ai[u] = 0.f;
+// One CTA per coarse site: the site's kept blocks are one (nq n) x n matrix
+// [row = (q, k)][j], read once in 16-byte pieces (VJ 2; odd n: VJ 1, rows start
+// on 8 bytes only).  Thread (ks, jp) takes VJ columns jp of the rows ks, ks + KS,
+// ... for RB right-hand sides at a time; the neighbours' vectors sit in shared
+// memory and the KS partial sums are added there in a fixed order.  Bound by the
+// blocks' stream (L2 between the products of one polynomial, when they fit).
+// One warp per site instead leaves 512 sites on 152 SMs to the latency of a serial
+// loop over all rows: 16^3 x 32, Nvec 40, 4 right-hand sides, order 8 took 2451 us
+// a call that way (345 us a product), 171 us this way, calls and copies included;
+// the blocks (59 MB) need 9 us a product from HBM.
+//
+// STEP 0: y = Q x + shift x.  STEP 1, 2: the Chebyshev step on d = x fused in:
+// y += d, s -= Q d, d' = c1 d + c2 s (d' to its own array: other sites still
+// read d); STEP 2, the last one, also adds d' to y and leaves max(|Re y|, |Im y|)
+// of each right-hand side in xm (cleared beforehand; may be null).
+struct QtArgs {
+  const float2* A9;
+  const int* nb9;
+  const float2* x;
+  float2* y;
+  float2* s;
+  float2* dn;
+  const int* skip;
+  unsigned* xm;
+  int nq, n, R;
+  float shift, c1, c2;
+};
+constexpr int QT_THREADS = 288;
+__host__ __device__ constexpr int qt_ks(int n, int VJ) { return QT_THREADS / ((n + VJ - 1) / VJ); }
+
+template <int VJ, int RB, int STEP>
+__global__ void __launch_bounds__(QT_THREADS) k_qtrunc_apply(const QtArgs g) {
+  extern __shared__ float2 qsm[];
+  if (g.skip && *g.skip) return;
+  const size_t a = blockIdx.x;
+  const int n = g.n, R = g.R, rows = g.nq * n;
+  const int NJ = (n + VJ - 1) / VJ, KS = qt_ks(n, VJ);
+  const int jp = threadIdx.x % NJ, ks = threadIdx.x / NJ;
+  float2* xs = qsm;                       // [row][RB]
+  float2* part = qsm + (size_t)rows * RB;   // [ks][j][RB]
+  const float2* A = g.A9 + a * 9 * (size_t)n * n;
+  for (int r0 = 0; r0 < R; r0 += RB) {
+    const int rb = min(RB, R - r0);
+    __syncthreads();
+    for (int i = threadIdx.x; i < rows * RB; i += QT_THREADS) {
+      const int row = i / RB, r = i % RB;
+      const size_t b = (size_t)__ldg(g.nb9 + a * 9 + row / n);
+      xs[i] = r < rb ? __ldg(g.x + (b * n + row % n) * R + r0 + r) : make_float2(0.f, 0.f);
     }
-    for (int q = 0; q < nq; ++q) {
-      const size_t b = (size_t)__ldg(nb9 + a * 9 + q);
-      const float2* blk = A9 + (a * 9 + q) * (size_t)n * n;
-      const float2* xb = x + b * (size_t)nout;
-#pragma unroll 4
-      for (int k = 0; k < n; ++k) {
+    __syncthreads();
+    float2 acc[VJ][RB];
+#pragma unroll
+    for (int v = 0; v < VJ; ++v)
+#pragma unroll
+      for (int r = 0; r < RB; ++r) acc[v][r] = make_float2(0.f, 0.f);
+    if (ks < KS) {
+      constexpr int U = 4;
+      for (int row = ks; row < rows; row += U * KS) {
+        float m[U][2 * VJ];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-          if (live[u]) {
-            const float2 m = __ldg(blk + k * n + jo[u]);
-            const float2 v = __ldg(xb + k * R + ro[u]);
-            ar[u] += m.x * v.x - m.y * v.y;
-            ai[u] += m.x * v.y + m.y * v.x;
+          const int k = row + u * KS;
+          const bool on = k < rows;
+          if constexpr (VJ == 2) {
+            const float4 q = on ? __ldg(reinterpret_cast<const float4*>(A + (size_t)k * n) + jp) : make_float4(0.f, 0.f, 0.f, 0.f);
+            m[u][0] = q.x; m[u][1] = q.y; m[u][2] = q.z; m[u][3] = q.w;
+          } else {
+            const float2 q = on ? __ldg(A + (size_t)k * n + jp) : make_float2(0.f, 0.f);
+            m[u][0] = q.x; m[u][1] = q.y;
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int k = min(row + u * KS, rows - 1);
+#pragma unroll
+          for (int r = 0; r < RB; ++r) {
+            const float2 x = xs[k * RB + r];
+#pragma unroll
+            for (int v = 0; v < VJ; ++v) {
+              acc[v][r].x = fmaf(m[u][2 * v], x.x, acc[v][r].x);
+              acc[v][r].y = fmaf(m[u][2 * v], x.y, acc[v][r].y);
+              acc[v][r].x = fmaf(-m[u][2 * v + 1], x.y, acc[v][r].x);
+              acc[v][r].y = fmaf(m[u][2 * v + 1], x.x, acc[v][r].y);
+            }
           }
         }
       }
-    }
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-      if (live[u]) {
-        const size_t o = a * (size_t)nout + o0 + lane + 32 * u;
-        const float2 v = x[o];
-        y[o] = make_float2(ar[u] + shift * v.x, ai[u] + shift * v.y);
+      for (int v = 0; v < VJ; ++v)
+#pragma unroll
+        for (int r = 0; r < RB; ++r) part[((size_t)ks * n + jp * VJ + v) * RB + r] = acc[v][r];
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < n * RB; i += QT_THREADS) {
+      const int j = i / RB, r = i % RB;
+      float2 q = make_float2(0.f, 0.f);
+      for (int k = 0; k < KS; ++k) {
+        const float2 p = part[(size_t)k * n * RB + i];
+        q.x += p.x;
+        q.y += p.y;
       }
+      float mx = 0.f;
+      if (r < rb) {
+        const size_t o = (a * n + j) * R + r0 + r;
+        const float2 d = g.x[o];
+        q.x += g.shift * d.x;
+        q.y += g.shift * d.y;
+        if (STEP == 0) {
+          g.y[o] = q;
+        } else {
+          float2 y = g.y[o], s = g.s[o], e;
+          y.x += d.x;
+          y.y += d.y;
+          s.x -= q.x;
+          s.y -= q.y;
+          e.x = g.c1 * d.x + g.c2 * s.x;
+          e.y = g.c1 * d.y + g.c2 * s.y;
+          if (STEP == 2) {
+            y.x += e.x;
+            y.y += e.y;
+            mx = fmaxf(fabsf(y.x), fabsf(y.y));
+          } else {
+            g.s[o] = s;
+            g.dn[o] = e;
+          }
+          g.y[o] = y;
+        }
+      }
+      if (STEP == 2 && g.xm && mx > 0.f) atomicMax(g.xm + r0 + r, __float_as_uint(mx));
     }
   }
 }
@@ -93,25 +171,6 @@ __global__ void k_cheb_init(const float2* __restrict__ r, float2* d, float2* s, 
   d[t] = make_float2(itheta * v.x, itheta * v.y);
   s[t] = v;
   y[t] = make_float2(0.f, 0.f);
-}
-
-// y += d; s -= q; d = c1 d + c2 s
-__global__ void k_cheb_step(float2* y, float2* s, float2* d, const float2* __restrict__ q, size_t n, float c1, float c2,
-                            const int* skip) {
-  if (skip && *skip) return;
-  const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= n) return;
-  float2 yv = y[t], sv = s[t], dv = d[t];
-  const float2 qv = q[t];
-  yv.x += dv.x;
-  yv.y += dv.y;
-  sv.x -= qv.x;
-  sv.y -= qv.y;
-  dv.x = c1 * dv.x + c2 * sv.x;
-  dv.y = c1 * dv.y + c2 * sv.y;
-  y[t] = yv;
-  s[t] = sv;
-  d[t] = dv;
 }
 
 // y += d; with xm != null, max(|Re y|, |Im y|) of each right-hand side into xm
@@ -197,21 +256,43 @@ __global__ void k_pow_norm(const float2* __restrict__ w, float2* v, size_t n, co
 
 }  // namespace
 
-void qtrunc_apply(Ctx& c, const Coarse& A, int R, const float2* x, float2* y, double shift, const int* skip) {
-  const QTrunc& Q = A.qt;
-  const int nout = A.nvec * R;
-  const unsigned grid = (unsigned)((A.Vc + 7) / 8);
-  if (nout <= 32)
-    k_qtrunc_apply_w<1><<<grid, 256, 0, c.stream>>>(Q.A9.as<float2>(), Q.nb9.as<int>(), Q.nq, A.nvec, x, R,
-                                                   (float)shift, y, skip, A.Vc);
-  else if (nout <= 64)
-    k_qtrunc_apply_w<2><<<grid, 256, 0, c.stream>>>(Q.A9.as<float2>(), Q.nb9.as<int>(), Q.nq, A.nvec, x, R,
-                                                   (float)shift, y, skip, A.Vc);
-  else
-    k_qtrunc_apply_w<4><<<grid, 256, 0, c.stream>>>(Q.A9.as<float2>(), Q.nb9.as<int>(), Q.nq, A.nvec, x, R,
-                                                   (float)shift, y, skip, A.Vc);
+template <int VJ, int RB, int STEP>
+static void launch_qtrunc(Ctx& c, const Coarse& A, const QtArgs& g) {
+  const size_t sm = ((size_t)g.nq * g.n + (size_t)qt_ks(g.n, VJ) * g.n) * RB * sizeof(float2);
+  auto fn = k_qtrunc_apply<VJ, RB, STEP>;
+  if (sm > 48 * 1024)
+    HDCG_CUDA(cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+  fn<<<(unsigned)A.Vc, QT_THREADS, sm, c.stream>>>(g);
   HDCG_CUDA(cudaGetLastError());
   ++c.launches;
+}
+
+// Right-hand sides per pass over the blocks: 1, 4 or 8.  A second pass re-reads a
+// site's blocks from L1 / L2; 16 accumulator sets would halve the resident warps.
+template <int STEP>
+static void dispatch_qtrunc(Ctx& c, const Coarse& A, QtArgs g) {
+  const bool vec = g.n % 2 == 0;
+  if (g.R == 1) vec ? launch_qtrunc<2, 1, STEP>(c, A, g) : launch_qtrunc<1, 1, STEP>(c, A, g);
+  else if (g.R <= 4) vec ? launch_qtrunc<2, 4, STEP>(c, A, g) : launch_qtrunc<1, 4, STEP>(c, A, g);
+  else vec ? launch_qtrunc<2, 8, STEP>(c, A, g) : launch_qtrunc<1, 8, STEP>(c, A, g);
+}
+
+static QtArgs qtrunc_args(const Coarse& A, int R, const float2* x, float2* y, double shift, const int* skip) {
+  QtArgs g{};
+  g.A9 = A.qt.A9.as<float2>();
+  g.nb9 = A.qt.nb9.as<int>();
+  g.x = x;
+  g.y = y;
+  g.skip = skip;
+  g.nq = A.qt.nq;
+  g.n = A.nvec;
+  g.R = R;
+  g.shift = (float)shift;
+  return g;
+}
+
+void qtrunc_apply(Ctx& c, const Coarse& A, int R, const float2* x, float2* y, double shift, const int* skip) {
+  dispatch_qtrunc<0>(c, A, qtrunc_args(A, R, x, y, shift, skip));
 }
 
 // y = M r for R right-hand sides (FP32 [e][r]); xm (nullable, cleared here)
@@ -221,22 +302,29 @@ void qtrunc_precondition(Ctx& c, Coarse& A, int R, const float2* r, float2* y, u
   const size_t ne = A.Vc * A.nvec, nc = ne * R;
   Q.work.ensure(3 * nc * sizeof(float2));
   float2* s = Q.work.as<float2>();
-  float2* d = s + nc;
-  float2* t = d + nc;
+  float2* d[2] = {s + nc, s + 2 * nc};   // the direction and the next one
   const double theta = 0.5 * (Q.hi + Q.lo), delta = 0.5 * (Q.hi - Q.lo);
-  const unsigned g = nblk(nc);
   if (xm) HDCG_CUDA(cudaMemsetAsync(xm, 0, RMAX * sizeof(unsigned), c.stream));
-  k_cheb_init<<<g, 256, 0, c.stream>>>(r, d, s, y, nc, (float)(1.0 / theta), skip);
+  k_cheb_init<<<nblk(nc), 256, 0, c.stream>>>(r, d[0], s, y, nc, (float)(1.0 / theta), skip);
+  ++c.launches;
   double rho = delta / theta;
   for (int k = 0; k + 1 < Q.order; ++k) {
-    qtrunc_apply(c, A, R, d, t, Q.shift, skip);
     const double rn = 1.0 / (2.0 * theta / delta - rho);
-    k_cheb_step<<<g, 256, 0, c.stream>>>(y, s, d, t, nc, (float)(rn * rho), (float)(2.0 * rn / delta), skip);
+    QtArgs g = qtrunc_args(A, R, d[k & 1], y, Q.shift, skip);
+    g.s = s;
+    g.dn = d[(k & 1) ^ 1];
+    g.c1 = (float)(rn * rho);
+    g.c2 = (float)(2.0 * rn / delta);
+    g.xm = xm;
+    if (k + 2 < Q.order) dispatch_qtrunc<1>(c, A, g);
+    else dispatch_qtrunc<2>(c, A, g);
     rho = rn;
   }
-  k_cheb_last<<<nblk(ne), 256, 0, c.stream>>>(y, d, ne, R, xm, skip);
+  if (Q.order == 1) {   // no product: y = d
+    k_cheb_last<<<nblk(ne), 256, 0, c.stream>>>(y, d[0], ne, R, xm, skip);
+    ++c.launches;
+  }
   HDCG_CUDA(cudaGetLastError());
-  c.launches += 2 + std::max(0, Q.order - 1);
 }
 
 void qtrunc_setup(Ctx& c, Coarse& A, int order, double lo, double hi, double shift) {
