@@ -73,6 +73,8 @@ __global__ void k_int_to_canon(const uint4* __restrict__ in, void* __restrict__ 
   for (int i = 0; i < 24; ++i) Canon<CT>::st(canon, t * 24 + i, (double)v[i]);
 }
 
+static unsigned blocks_for(size_t n) { return (unsigned)((n + 255) / 256); }
+
 // Canonical and internal fields of one element type hold the same 16-byte
 // granules, canonical [site][chunk], internal [chunk][site]: a transposition
 // through shared memory, with whole granules coalesced on both sides.  Bound by
@@ -131,6 +133,25 @@ __global__ void __launch_bounds__(256) k_granules(const uint4* __restrict__ src,
   }
 }
 
+// 16-bit fields: a site's 48 bytes hold the twelve complex numbers as
+// [spin][colour] in the canonical and as [colour][spin] in the internal layout
+template <bool IN>
+__global__ void __launch_bounds__(256) k_words(const uint4* __restrict__ src, uint4* __restrict__ dst, size_t n) {
+  const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= n) return;
+  unsigned w[12], o[12];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) *reinterpret_cast<uint4*>(w + 4 * c) = __ldg(src + 3 * t + c);
+#pragma unroll
+  for (int i = 0; i < 12; ++i) {
+    const int j = IN ? 3 * (i % 4) + i / 4 : 4 * (i % 3) + i / 3;
+    o[i] = w[j];
+  }
+#pragma unroll
+  for (int c = 0; c < 3; ++c)
+    dst[3 * t + c] = make_uint4(o[4 * c], o[4 * c + 1], o[4 * c + 2], o[4 * c + 3]);
+}
+
 // true if the transposition ran: same element type on both sides and 16-byte
 // aligned buffers (a caller's canonical pointer may be aligned to its element only)
 template <bool IN, typename CV>
@@ -140,7 +161,7 @@ static bool launch_granules(Ctx& c, int bytes, const void* src, void* dst, size_
   const uint4* s = reinterpret_cast<const uint4*>(src);
   uint4* d = reinterpret_cast<uint4*>(dst);
   auto grid = [&](int ts) { return dim3((unsigned)((c.n5 + ts - 1) / ts), (unsigned)nf); };
-  if (bytes == 2) k_granules<3, IN, CV><<<grid(granule_tile<3>()), 256, 0, c.stream>>>(s, d, c.n5);
+  if (bytes == 2) k_words<IN><<<blocks_for(c.n5 * nf), 256, 0, c.stream>>>(s, d, c.n5 * nf);
   else if (bytes == 4) k_granules<6, IN, CV><<<grid(granule_tile<6>()), 256, 0, c.stream>>>(s, d, c.n5);
   else k_granules<12, IN, CV><<<grid(granule_tile<12>()), 256, 0, c.stream>>>(s, d, c.n5);
   HDCG_CUDA(cudaGetLastError());
@@ -166,8 +187,6 @@ __global__ void k_convert(const uint4* __restrict__ in, uint4* __restrict__ out,
   for (int i = 0; i < 24; ++i) w[i] = (Ro)v[i];
   store_spinor<So, Ro>(out + f * n5 * Store<So>::chunks, site5, n5, w);
 }
-
-static unsigned blocks_for(size_t n) { return (unsigned)((n + 255) / 256); }
 
 void canon_to_internal(Ctx& c, const void* canon, int canon_prec, uint4* out, int prec, size_t nf) {
   const unsigned g = blocks_for(c.n5 * nf);

@@ -165,11 +165,11 @@ __device__ void load_tile(Rt* sm, const uint4* base, size_t kstride, int nv, con
     const int ch = (q / TILE) % C;
     const int k = q / (C * TILE);
     const size_t site5 = block_site5(ba, b, tile0 + t);
-    const uint4 g = __ldg(base + k * kstride + ch * ba.n5 + site5);
+    const uint4 g = __ldg(base + k * kstride + granule_at<S>(ch, site5, ba.n5));
     R tmp[P];
     unpack(S{}, g, tmp);
 #pragma unroll
-    for (int i = 0; i < P; ++i) sm[k * TROW + t * 24 + ch * P + i] = (Rt)tmp[i];
+    for (int i = 0; i < P; ++i) sm[k * TROW + t * 24 + real_of<S>(ch, i)] = (Rt)tmp[i];
   }
 }
 
@@ -186,8 +186,8 @@ __device__ void store_tile(const Rt* sm, uint4* base, size_t kstride, int nv, co
     const size_t site5 = block_site5(ba, b, tile0 + t);
     R tmp[P];
 #pragma unroll
-    for (int i = 0; i < P; ++i) tmp[i] = (R)sm[k * TROW + t * 24 + ch * P + i];
-    base[k * kstride + ch * ba.n5 + site5] = pack(S{}, tmp);
+    for (int i = 0; i < P; ++i) tmp[i] = (R)sm[k * TROW + t * 24 + real_of<S>(ch, i)];
+    base[k * kstride + granule_at<S>(ch, site5, ba.n5)] = pack(S{}, tmp);
   }
 }
 
@@ -284,17 +284,18 @@ __global__ void __launch_bounds__(256) k_block_transform(uint4* X, size_t xstrid
       for (int i = 0; i < P; ++i) o[i] = 0;
       for (int j = 0; j <= k && j < n; ++j) {
         const Rt tr = ts[2 * (j * n + k)], ti = ts[2 * (j * n + k) + 1];
-        const Rt* xr = xs + j * TROW + t * 24 + ch * P;
+        const Rt* xr = xs + j * TROW + t * 24;
 #pragma unroll
         for (int i = 0; i < P; i += 2) {
-          o[i] += xr[i] * tr - xr[i + 1] * ti;
-          o[i + 1] += xr[i] * ti + xr[i + 1] * tr;
+          const Rt xre = xr[real_of<S>(ch, i)], xim = xr[real_of<S>(ch, i) + 1];
+          o[i] += xre * tr - xim * ti;
+          o[i + 1] += xre * ti + xim * tr;
         }
       }
       R w[P];
 #pragma unroll
       for (int i = 0; i < P; ++i) w[i] = (R)o[i];
-      X[k * xstride + ch * ba.n5 + block_site5(ba, b, tile0 + t)] = pack(S{}, w);
+      X[k * xstride + granule_at<S>(ch, block_site5(ba, b, tile0 + t), ba.n5)] = pack(S{}, w);
     }
   }
 }
@@ -1434,8 +1435,7 @@ __global__ void __launch_bounds__(256) k_prolong_multi(const uint4* phi, size_t 
                                                        const double* un_num, const double* un_den) {
   using Ro = typename Store<So>::real;
   using Ra = typename Store<Sa>::real;
-  constexpr int C = Store<So>::chunks, P = Store<So>::per_chunk, PA = Store<Sa>::per_chunk;
-  static_assert(PA >= P, "the added field's chunks hold at least one output chunk");
+  constexpr int C = Store<So>::chunks, P = Store<So>::per_chunk;
   extern __shared__ __align__(16) unsigned char smraw[];
   Rt* xs = reinterpret_cast<Rt*>(smraw);
   Rt* cs = xs + (size_t)n * TROW;    // [k][r] complex
@@ -1463,27 +1463,39 @@ __global__ void __launch_bounds__(256) k_prolong_multi(const uint4* phi, size_t 
       for (int i = 0; i < P; ++i) o[i] = 0;
       for (int k = 0; k < n; ++k) {
         const Rt cr = cs[2 * (k * R + r)], ci = cs[2 * (k * R + r) + 1];
-        const Rt* xr = xs + k * TROW + t * 24 + ch * P;
+        const Rt* xr = xs + k * TROW + t * 24;
 #pragma unroll
         for (int i = 0; i < P; i += 2) {
-          o[i] += cr * xr[i] - ci * xr[i + 1];
-          o[i + 1] += cr * xr[i + 1] + ci * xr[i];
+          const Rt xre = xr[real_of<So>(ch, i)], xim = xr[real_of<So>(ch, i) + 1];
+          o[i] += cr * xre - ci * xim;
+          o[i + 1] += cr * xim + ci * xre;
         }
       }
       const size_t site5 = block_site5(ba, b, tile0 + t);
       if (add) {
-        // the P reals of this output chunk sit in chunk (ch P) / PA of the added field
-        Ra av[PA];
-        unpack(Sa{}, __ldg(add + r * astride + ((ch * P) / PA) * ba.n5 + site5), av);
-        const int off = (ch * P) % PA;
+        if constexpr (std::is_same<So, Sa>::value) {
+          Ra av[P];
+          unpack(Sa{}, __ldg(add + r * astride + granule_at<Sa>(ch, site5, ba.n5)), av);
 #pragma unroll
-        for (int i = 0; i < P; ++i) o[i] += (Rt)av[off + i];
+          for (int i = 0; i < P; ++i) o[i] += (Rt)av[i];
+        } else {
+          // FP16 added to FP32 or FP64: one 32-bit word (spin, colour) per complex number
+          static_assert(std::is_same<Sa, f16_t>::value && Store<So>::chunks != 3, "the added field is FP16");
+          const unsigned* words = reinterpret_cast<const unsigned*>(add + r * astride) + site5 * 12;
+#pragma unroll
+          for (int i = 0; i < P; i += 2) {
+            const int z = (ch * P + i) / 2;                      // spin * 3 + colour
+            const float2 av = h2f(__ldg(words + 4 * (z % 3) + z / 3));
+            o[i] += (Rt)av.x;
+            o[i + 1] += (Rt)av.y;
+          }
+        }
       }
       const Rt f = unscale[r];
       Ro w[P];
 #pragma unroll
       for (int i = 0; i < P; ++i) w[i] = (Ro)(f * o[i]);
-      out[r * ostride + ch * ba.n5 + site5] = pack(So{}, w);
+      out[r * ostride + granule_at<So>(ch, site5, ba.n5)] = pack(So{}, w);
     }
   }
 }

@@ -5,9 +5,13 @@
 // (site5 = cb4 * Ls + s; reals ordered [spin][colour][re, im]) are split into
 // 16-byte chunks, and chunk c of every site is stored contiguously:
 //   field[c * n5 + site5]  (uint4 granules).
-// FP64: 12 chunks of 2 doubles, FP32: 6 chunks of 4 floats, 16-bit: 3 chunks
-// of 8 halves.  Consecutive threads (consecutive s, then sites) therefore
-// load consecutive 16-byte granules.
+// FP64: 12 chunks of 2 doubles, FP32: 6 chunks of 4 floats.  Consecutive
+// threads (consecutive s, then sites) therefore load consecutive 16-byte granules.
+//
+// 16-bit storage: 3 chunks of 8 halves, chunk c holding colour c of the four
+// spins, and a site's chunks are contiguous: field[site5 * 3 + c].  That is the
+// order of the tensor-core hop's operand (hop_tc.cuh): lanes of neighbouring
+// slices and of the three colours read one contiguous run.
 #pragma once
 
 #include <cuda_bf16.h>
@@ -129,6 +133,17 @@ __device__ __forceinline__ uint4 pack(bf16t_t, const float* r) {
   return make_uint4(f2b2t(r[0], r[1]), f2b2t(r[2], r[3]), f2b2t(r[4], r[5]), f2b2t(r[6], r[7]));
 }
 
+// granule c of site site5, and the canonical index ([spin][colour][re, im]) of
+// the i-th real in granule c
+template <typename St>
+__device__ __forceinline__ size_t granule_at(int c, size_t site5, size_t n5) {
+  return Store<St>::chunks == 3 ? site5 * 3 + c : c * n5 + site5;
+}
+template <typename St>
+__host__ __device__ constexpr int real_of(int c, int i) {
+  return Store<St>::chunks == 3 ? 2 * (3 * (i / 2) + c) + (i & 1) : c * Store<St>::per_chunk + i;
+}
+
 // whole-spinor load / store in the chunked layout ------------------------------
 template <typename St, typename R>
 __device__ __forceinline__ void load_spinor(const uint4* __restrict__ f, size_t site5, size_t n5,
@@ -136,11 +151,11 @@ __device__ __forceinline__ void load_spinor(const uint4* __restrict__ f, size_t 
   constexpr int C = Store<St>::chunks, P = Store<St>::per_chunk;
 #pragma unroll
   for (int c = 0; c < C; ++c) {
-    uint4 g = __ldg(f + c * n5 + site5);
+    uint4 g = __ldg(f + granule_at<St>(c, site5, n5));
     typename Store<St>::real t[P];
     unpack(St{}, g, t);
 #pragma unroll
-    for (int i = 0; i < P; ++i) v[c * P + i] = (R)t[i];
+    for (int i = 0; i < P; ++i) v[real_of<St>(c, i)] = (R)t[i];
   }
 }
 
@@ -152,8 +167,8 @@ __device__ __forceinline__ void store_spinor(uint4* __restrict__ f, size_t site5
   for (int c = 0; c < C; ++c) {
     typename Store<St>::real t[P];
 #pragma unroll
-    for (int i = 0; i < P; ++i) t[i] = (typename Store<St>::real)v[c * P + i];
-    f[c * n5 + site5] = pack(St{}, t);
+    for (int i = 0; i < P; ++i) t[i] = (typename Store<St>::real)v[real_of<St>(c, i)];
+    f[granule_at<St>(c, site5, n5)] = pack(St{}, t);
   }
 }
 

@@ -19,6 +19,7 @@
 // read once per CTA group and reused by its Ls lanes (Sec. 6.5: Ls-fold link reuse).
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <vector>
 
@@ -63,6 +64,7 @@ __global__ void nbr_kernel(Geom g, int* nbr) {
   }
 }
 
+// 16-bit links: rows of three, each padded to a 16-byte granule.
 // links[p][i][dir][3][3]: dir < 4: U_mu(x); dir >= 4: U_mu(x - mu)^dag; the
 // antiperiodic time boundary is folded in as a sign.
 __global__ void link_kernel(Geom g, int apbc, const double2* __restrict__ U, double2* l64,
@@ -91,8 +93,8 @@ __global__ void link_kernel(Geom g, int apbc, const double2* __restrict__ U, dou
         const int e = r * 3 + c;
         l64[(i * 8 + dir) * 9 + e] = v;
         l32[(i * 8 + dir) * 10 + e] = make_float2((float)v.x, (float)v.y);
-        l16[(i * 8 + dir) * 12 + e] = __floats2half2_rn((float)v.x, (float)v.y);
-        lb16[(i * 8 + dir) * 12 + e] = __floats2bfloat162_rn((float)v.x, (float)v.y);
+        l16[(i * 8 + dir) * 12 + 4 * r + c] = __floats2half2_rn((float)v.x, (float)v.y);
+        lb16[(i * 8 + dir) * 12 + 4 * r + c] = __floats2bfloat162_rn((float)v.x, (float)v.y);
         const float rh = __double2float_rn(v.x), ih = __double2float_rn(v.y);
         ldf[(i * 8 + dir) * 9 + e] =
             make_float4(rh, __double2float_rn(v.x - (double)rh), ih, __double2float_rn(v.y - (double)ih));
@@ -268,6 +270,20 @@ static int hop_threads(const Ctx& c, int prec, int nrhs) {
   return c.n5 * (size_t)nrhs < (size_t)152 * 256 * 2 ? 64 : 256;
 }
 
+// 16-bit storage with Ls >= 8 runs on the tensor cores unless a variant is
+// forced: a warp's 16 rows are slices of one 4D site (half of them at Ls 8).
+// Faster there at every size measured (hop_tc.cuh); at Ls 4 and 2 a quarter or an
+// eighth of the rows would be filled, and the scalar kernel's work is per slice.
+static bool hop_use_tc(const Ctx& c, int prec) {
+  return is_16bit(prec) && c.hop_force < 0 && c.Ls >= 8;
+}
+
+// persistent: as many CTAs as are resident, each warp striding over the sites
+static unsigned hop_tc_grid(const Ctx& c) {
+  const size_t ctas = (c.n4 + tch::TC_WARPS - 1) / tch::TC_WARPS;
+  return (unsigned)std::min<size_t>(ctas, 152 * tch::tc_ctas(c.Ls / 8));
+}
+
 void launch_hop(Ctx& c, int pass, int prec, const uint4* in, const uint4* in2, uint4* out,
                 const HopEpi& epi, double* red_result, int accumulate) {
   HDCG_REQUIRE(c.have_gauge && c.have_dwf, HDCG_ERR_STATE, "gauge field and DWF parameters required");
@@ -313,8 +329,9 @@ void launch_hop(Ctx& c, int pass, int prec, const uint4* in, const uint4* in2, u
   a.al_lam = epi.al_lam;
   a.fstride = epi.nrhs > 1 ? epi.fstride : 0;
   a.al_mask = epi.mask;
+  const bool tc = hop_use_tc(c, prec);
   const int threads = hop_threads(c, prec, epi.nrhs);
-  const unsigned grid = (unsigned)((c.n5 + threads - 1) / threads);
+  const unsigned grid = tc ? hop_tc_grid(c) : (unsigned)((c.n5 + threads - 1) / threads);
   HDCG_REQUIRE(epi.nrhs >= 1 && epi.nrhs <= RMAX, HDCG_ERR_ARG, "1 <= right-hand sides <= 16");
   a.do_red = red_result != nullptr;
   if (a.do_red) {
@@ -327,7 +344,7 @@ void launch_hop(Ctx& c, int pass, int prec, const uint4* in, const uint4* in2, u
   }
   const bool mob = c.co.c != 0.0;
   const dim3 grid2(grid, (unsigned)epi.nrhs);
-  const int v = hop_variant(c, prec, pass, mob, a, grid2, threads);
+  const int v = tc ? HOP_TC : hop_variant(c, prec, pass, mob, a, grid2, threads);
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
   if (c.prof.on) {
     HDCG_CUDA(cudaEventCreate(&ev0));

@@ -111,7 +111,8 @@ __device__ __forceinline__ void load_link16(const uint4* __restrict__ p, float* 
   }
 #pragma unroll
   for (int i = 0; i < 9; ++i) {
-    const float2 v = bf ? b2f(t[i]) : h2f(t[i]);
+    const unsigned e = t[4 * (i / 3) + i % 3];   // rows of three, padded to a granule
+    const float2 v = bf ? b2f(e) : h2f(e);
     u[2 * i] = v.x;
     u[2 * i + 1] = v.y;
   }
@@ -381,7 +382,7 @@ __device__ __forceinline__ void hop_raw(const HopArgs& a, const uint4 (&raw)[8][
       float t[8];
       unpack(St{}, raw[MU + 4 * side][c], t);
 #pragma unroll
-      for (int i = 0; i < 8; ++i) ps[c * 8 + i] = (R)t[i];
+      for (int i = 0; i < 8; ++i) ps[real_of<St>(c, i)] = (R)t[i];
     }
     if (KIN) apply_lin<R, false>(ps, sc<R>(a.b, a.fb, a.lb), sc<R>(a.c, a.fc, a.lc), s, a.Ls, sc<R>(a.mass, a.fmass, a.lmass));
     R h[12], uh[12], U[18];
@@ -402,6 +403,18 @@ __device__ __forceinline__ void hop_raw(const HopArgs& a, const uint4 (&raw)[8][
 // warp sums its lanes' float partials by double-float TwoSum steps on the FP32
 // pipes (about 48 bits) and only the per-warp totals are added in FP64; the
 // FP64 and double-float passes reduce in FP64 throughout.
+__device__ __forceinline__ void norm2_reduce(float hi, float lo, const Reduction& red) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const float oh = __shfl_xor_sync(FULL_MASK, hi, o), ol = __shfl_xor_sync(FULL_MASK, lo, o);
+    float sh, eh;
+    two_sum(hi, oh, sh, eh);
+    eh = __fadd_rn(eh, __fadd_rn(lo, ol));
+    fast_two_sum(sh, eh, hi, lo);
+  }
+  double v[1] = {(double)hi + (double)lo};
+  grid_reduce<1, true>(v, red);
+}
 template <typename R>
 __device__ __forceinline__ void hop_norm2(const R* acc, bool active, const Reduction& red) {
   if constexpr (std::is_same<R, float>::value) {
@@ -410,17 +423,7 @@ __device__ __forceinline__ void hop_norm2(const R* acc, bool active, const Reduc
 #pragma unroll
       for (int i = 0; i < 24; ++i) t = fmaf(acc[i], acc[i], t);
     }
-    float hi = t, lo = 0.f;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const float oh = __shfl_xor_sync(FULL_MASK, hi, o), ol = __shfl_xor_sync(FULL_MASK, lo, o);
-      float sh, eh;
-      two_sum(hi, oh, sh, eh);
-      eh = __fadd_rn(eh, __fadd_rn(lo, ol));
-      fast_two_sum(sh, eh, hi, lo);
-    }
-    double v[1] = {(double)hi + (double)lo};
-    grid_reduce<1, true>(v, red);
+    norm2_reduce(t, 0.f, red);
   } else {
     double nrm2 = 0.0;
     if (active) {
@@ -491,7 +494,7 @@ __global__ void __launch_bounds__(hop_bound<St>(), hop_ctas<St, MINB>()) hop_ker
 #pragma unroll
     for (int d = 0; d < 8; ++d)
 #pragma unroll
-      for (int c = 0; c < 3; ++c) raw[d][c] = __ldg(in + c * a.n5 + (size_t)nbv[d] * a.Ls + s);
+      for (int c = 0; c < 3; ++c) raw[d][c] = __ldg(in + granule_at<St>(c, (size_t)nbv[d] * a.Ls + s, a.n5));
     hop_raw<St, R, LT, 0, SF, PASS == PASS_A && MOB>(a, raw, lk, s, acc);
     hop_raw<St, R, LT, 1, SF, PASS == PASS_A && MOB>(a, raw, lk, s, acc);
     hop_raw<St, R, LT, 2, SF, PASS == PASS_A && MOB>(a, raw, lk, s, acc);
@@ -586,6 +589,7 @@ __global__ void __launch_bounds__(hop_bound<St>(), hop_ctas<St, MINB>()) hop_ker
 }  // namespace hdcg
 
 #include "hop_packed.cuh"
+#include "hop_tc.cuh"
 
 namespace hdcg {
 
@@ -593,11 +597,15 @@ namespace hdcg {
 // double-float arithmetic for FP64 storage; 5th and 6th (FP32 and 16-bit
 // storage only): packed FP32 arithmetic (hop_packed.cuh) with MINB 2 and 1
 constexpr int HOP_VARIANTS = 6;
+constexpr int HOP_TC = 6;   // the tensor-core pass (16-bit storage, Ls >= 8)
 template <typename St> constexpr int hop_variants() { return Store<St>::chunks == 12 ? 4 : 6; }
 
 // launch variant v of one pass for storage St
 template <typename St>
 void launch_hop_variant(int v, int pass, bool mob, const HopArgs& a, dim3 grid, int threads, cudaStream_t st) {
+  if constexpr (Store<St>::chunks == 3) {
+    if (v == HOP_TC) return launch_hop_tc<St>(pass, mob, a, grid, st);
+  }
   if constexpr (Store<St>::chunks != 12) {
     if (v >= 4) {
       const bool stage = a.Ls >= 8;

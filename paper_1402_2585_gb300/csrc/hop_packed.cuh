@@ -91,13 +91,18 @@ template <typename St>
 __device__ __forceinline__ void load_raw(const uint4* __restrict__ f, size_t site5, size_t n5,
                                          uint4 (&g)[Store<St>::chunks]) {
 #pragma unroll
-  for (int c = 0; c < Store<St>::chunks; ++c) g[c] = __ldg(f + c * n5 + site5);
+  for (int c = 0; c < Store<St>::chunks; ++c) g[c] = __ldg(f + granule_at<St>(c, site5, n5));
 }
 template <typename St>
 __device__ __forceinline__ void unpack_site(const uint4 (&g)[Store<St>::chunks], c2* v) {
   constexpr int PC = Store<St>::per_chunk / 2;   // complex per granule
 #pragma unroll
-  for (int c = 0; c < Store<St>::chunks; ++c) unpack_c(St{}, g[c], v + c * PC);
+  for (int c = 0; c < Store<St>::chunks; ++c) {
+    c2 z[PC];
+    unpack_c(St{}, g[c], z);
+#pragma unroll
+    for (int i = 0; i < PC; ++i) v[real_of<St>(c, 2 * i) / 2] = z[i];
+  }
 }
 template <typename St>
 __device__ __forceinline__ void load_c(const uint4* __restrict__ f, size_t site5, size_t n5, c2* v) {
@@ -128,7 +133,12 @@ template <typename St>
 __device__ __forceinline__ void store_c(uint4* __restrict__ f, size_t site5, size_t n5, const c2* v) {
   constexpr int PC = Store<St>::per_chunk / 2;
 #pragma unroll
-  for (int c = 0; c < Store<St>::chunks; ++c) f[c * n5 + site5] = pack_c(St{}, v + c * PC);
+  for (int c = 0; c < Store<St>::chunks; ++c) {
+    c2 z[PC];
+#pragma unroll
+    for (int i = 0; i < PC; ++i) z[i] = v[real_of<St>(c, 2 * i) / 2];
+    f[granule_at<St>(c, site5, n5)] = pack_c(St{}, z);
+  }
 }
 
 // v <- a v + b P v (P_s, or P_s^dag for DAG; wall factor -m), see apply_lin
@@ -250,12 +260,12 @@ __device__ __forceinline__ float4 link_entry<float2>(const uint4* __restrict__ l
 }
 template <>
 __device__ __forceinline__ float4 link_entry<__half2>(const uint4* __restrict__ lk, int e) {
-  const float2 v = h2f(__ldg(reinterpret_cast<const unsigned*>(lk) + e));
+  const float2 v = h2f(__ldg(reinterpret_cast<const unsigned*>(lk) + 4 * (e / 3) + e % 3));
   return make_float4(v.x, v.x, -v.y, v.y);
 }
 template <>
 __device__ __forceinline__ float4 link_entry<__nv_bfloat162>(const uint4* __restrict__ lk, int e) {
-  const float2 v = b2f(__ldg(reinterpret_cast<const unsigned*>(lk) + e));
+  const float2 v = b2f(__ldg(reinterpret_cast<const unsigned*>(lk) + 4 * (e / 3) + e % 3));
   return make_float4(v.x, v.x, -v.y, v.y);
 }
 

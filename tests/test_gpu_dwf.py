@@ -144,3 +144,37 @@ def test_fused_cg_step_every_variant(variant):
     xg = x.cpu().numpy()
     assert np.sqrt(norm2(b - d.mdagm(xg)) / norm2(b)) <= 1.05e-9
     assert rel(xg, xs) < 1e-6
+
+
+@pytest.mark.parametrize("prec", [F16, BF16, BF16T])
+@pytest.mark.parametrize("dims,Ls,b,c,apbc", [((2, 2, 2, 2), 16, 1.0, 0.0, False), ((4, 2, 6, 4), 16, 1.5, 0.5, True),
+                                              ((2, 4, 2, 2), 32, 1.0, 0.0, True), ((4, 4, 2, 6), 32, 2.0, 1.0, False),
+                                              ((2, 2, 4, 2), 8, 1.0, 0.0, True), ((4, 6, 2, 4), 8, 1.5, 0.5, False)])
+def test_tensor_core_pass_against_the_scalar_pass(prec, dims, Ls, b, c, apbc):
+    """16-bit storage with Ls >= 8 runs on the tensor cores: every pass is as
+    far from the oracle as the scalar kernel (forced variant 0), within a tenth
+    (the error is that of the 16-bit links, inputs and intermediates, which both
+    round alike; FP32 rounding is 2^-13 of it)."""
+    torch = torch_or_skip()
+    U = sy.gauge_field(dims, 0.4, 700)
+    d = DWF(dims, Ls, 1.8, b, c, 0.02, U, antiperiodic_t=apbc)
+    h = Hdcg(dims, Ls, antiperiodic_t=apbc, stream=torch.cuda.current_stream().cuda_stream)
+    h.set_dwf(1.8, b, c, 0.02)
+    h.set_gauge(torch.from_numpy(U).cuda())
+    psi = sy.gaussian_fermion(dims, Ls, 701)
+    x = to_gpu(psi, prec)
+    err = {}
+    for variant in (0, -1):
+        h.set_hop_variant(variant)
+        y = torch.empty_like(x)
+        e = []
+        for dagger, ref in ((False, d.mpc), (True, d.mpc_dag)):
+            h.apply_mpc(x, y, dagger=dagger, prec=prec)
+            e.append(rel(from_gpu(y), ref(psi)))
+        pHp = h.apply_mdagm(x, y, prec=prec, want_pHp=True)
+        e.append(rel(from_gpu(y), d.mdagm(psi)))
+        assert pHp == pytest.approx(norm2(d.mpc(psi)), rel=TOL[prec])
+        err[variant] = e
+    for tc, scalar in zip(err[-1], err[0]):
+        assert tc < TOL[prec]
+        assert tc <= 1.1 * scalar
