@@ -20,6 +20,7 @@
 #include <vector>
 
 #include "coarse.cuh"
+#include "mma.cuh"
 
 namespace hdcg {
 
@@ -447,65 +448,261 @@ template <typename C> struct CV;
 template <> struct CV<float> { using T = float2; };
 template <> struct CV<double> { using T = double2; };
 
-constexpr int RKC = 16;  // subspace vectors per restriction pass
-
-template <typename Sp, typename Sv, typename Rc>
-__global__ void __launch_bounds__(256) k_restrict(const uint4* __restrict__ phi, size_t pstride, int nvec,
-                                                  const uint4* __restrict__ v, BlockArgs ba,
-                                                  typename CV<Rc>::T* out) {
-  using Rp = typename Store<Sp>::real;
-  using Rv = typename Store<Sv>::real;
-  using R = typename std::conditional<(sizeof(Rp) > sizeof(Rv)), Rp, Rv>::type;
-  const size_t b = blockIdx.x;
-  const int nsites = ba.spb * ba.Ls;
-  for (int k0 = 0; k0 < nvec; k0 += RKC) {
-    const int kc = min(RKC, nvec - k0);
-    R accr[2 * RKC];
-#pragma unroll
-    for (int q = 0; q < 2 * RKC; ++q) accr[q] = 0;
-    for (int g = threadIdx.x; g < nsites; g += blockDim.x) {
-      const size_t site5 = block_site5(ba, b, g);
-      Rv vv[24];
-      load_spinor<Sv, Rv>(v, site5, ba.n5, vv);
-#pragma unroll
-      for (int q = 0; q < RKC; ++q) {
-        if (q < kc) {
-          Rp pv[24];
-          load_spinor<Sp, Rp>(phi + (size_t)(k0 + q) * pstride, site5, ba.n5, pv);
-          R sr = 0, si = 0;
-#pragma unroll
-          for (int e = 0; e < 24; e += 2) {
-            sr += (R)pv[e] * (R)vv[e] + (R)pv[e + 1] * (R)vv[e + 1];
-            si += (R)pv[e] * (R)vv[e + 1] - (R)pv[e + 1] * (R)vv[e];
-          }
-          accr[2 * q] += sr;
-          accr[2 * q + 1] += si;
-        }
-      }
-    }
-    double acc[2 * RKC];
-#pragma unroll
-    for (int q = 0; q < 2 * RKC; ++q) acc[q] = (double)accr[q];
-    block_sum<2 * RKC>(acc);
-    if (threadIdx.x == 0)
-      for (int q = 0; q < kc; ++q) out[b * nvec + k0 + q] = {(Rc)acc[2 * q], (Rc)acc[2 * q + 1]};
-    __syncthreads();
+// complex number z (spin * 3 + colour) of site site5
+template <typename S>
+__device__ __forceinline__ void load_complex(const uint4* __restrict__ f, int z, size_t site5, size_t n5,
+                                             typename Store<S>::real& re, typename Store<S>::real& im) {
+  if constexpr (Store<S>::chunks == 3) {
+    const unsigned w = __ldg(reinterpret_cast<const unsigned*>(f) + site5 * 12 + 4 * (z % 3) + z / 3);
+    const float2 v = std::is_same<S, f16_t>::value ? h2f(w) : b2f(w);
+    re = v.x;
+    im = v.y;
+  } else if constexpr (Store<S>::chunks == 6) {
+    const uint2 w = __ldg(reinterpret_cast<const uint2*>(f + (size_t)(z / 2) * n5 + site5) + (z & 1));
+    re = __uint_as_float(w.x);
+    im = __uint_as_float(w.y);
+  } else {
+    typename Store<S>::real r[2];
+    unpack(S{}, __ldg(f + (size_t)z * n5 + site5), r);
+    re = r[0];
+    im = r[1];
   }
 }
 
-void restrict_field(Ctx& c, const Subspace& s, const uint4* v, int vprec, void* cvec, int cprec) {
-  const size_t pstride = s.vec_bytes(c) / 16;
+// a float as a double without the FP64 pipe's conversion
+__device__ __forceinline__ double widen(float x) {
+  double d;
+  return widen_float(x, d) ? d : (double)x;
+}
+__device__ __forceinline__ double widen(double x) { return x; }
+
+// Sums the 32 values of every lane over the warp: lane l returns the total of
+// v[l].  31 additions instead of 160 for a butterfly per value (the FP64 pipe
+// does two lanes per clock and SM).
+__device__ __forceinline__ double warp_scatter_sum(double (&v)[32]) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const bool up = lane & o;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      if (i < o) {
+        const double keep = up ? v[i + o] : v[i], send = up ? v[i] : v[i + o];
+        v[i] = keep + __shfl_xor_sync(FULL_MASK, send, o);
+      }
+    }
+  }
+  return v[0];
+}
+
+// c[b][k][r] = <phi_k^b, v_r>: one CTA per block (x) and group of KC vectors (y).  A thread owns granules of the
+// subspace's layout: RB fields' values of a granule stay in registers while the KC
+// vectors stream by in 16-byte loads, so lanes read consecutive granules in every
+// layout.  Thread sums are FP32 (FP64 with FP64 operands) over its granules, the
+// sums over threads FP64.  Bound by the stream of the vectors.  (One thread per
+// site with sums of 32 doubles per warp by butterflies: 2408 us for 24^3 x 48 x 16,
+// 32 FP16 vectors, 8.4 GB; both kernels of this file together now take 2.6 ms of
+// P R at that size, of 3.6.)
+template <typename Sp, typename Sv, typename Rc, int KC, int RB>
+__global__ void __launch_bounds__(256) k_restrict(const uint4* __restrict__ phi, size_t pstride, int nvec,
+                                                  const uint4* __restrict__ v, size_t vstride, int R, BlockArgs ba,
+                                                  typename CV<Rc>::T* out) {
+  static_assert(KC * RB == 16, "32 sums per thread");
+  using Rp = typename Store<Sp>::real;
+  using Rv = typename Store<Sv>::real;
+  using T = typename std::conditional<(sizeof(Rp) > sizeof(Rv)), Rp, Rv>::type;
+  constexpr int C = Store<Sp>::chunks, P = Store<Sp>::per_chunk;
+  __shared__ double part[8][32];
+  const size_t b = blockIdx.x;
+  const int k0 = blockIdx.y * KC, kc = min(KC, nvec - k0);
+  const int ng = ba.spb * ba.Ls * C;
+  for (int r0 = 0; r0 < R; r0 += RB) {
+    const int rb = min(RB, R - r0);
+    T acc[KC][RB][2];
+#pragma unroll
+    for (int k = 0; k < KC; ++k)
+#pragma unroll
+      for (int r = 0; r < RB; ++r) acc[k][r][0] = acc[k][r][1] = 0;
+    for (int i = threadIdx.x; i < ng; i += 256) {
+      // chunk-major storage: consecutive threads take consecutive sites of a chunk
+      const int ch = C == 3 ? i % 3 : i / (ba.spb * ba.Ls), g = C == 3 ? i / 3 : i % (ba.spb * ba.Ls);
+      const size_t site5 = block_site5(ba, b, g);
+      const uint4* pk = phi + k0 * pstride + granule_at<Sp>(ch, site5, ba.n5);
+      uint4 raw[KC];
+#pragma unroll
+      for (int k = 0; k < KC; ++k) raw[k] = __ldg(pk + (size_t)min(k, kc - 1) * pstride);
+      T vv[RB][P];
+#pragma unroll
+      for (int r = 0; r < RB; ++r)
+#pragma unroll
+        for (int e = 0; e < P; e += 2) {
+          Rv re = 0, im = 0;
+          if (r < rb) load_complex<Sv>(v + (r0 + r) * vstride, real_of<Sp>(ch, e) / 2, site5, ba.n5, re, im);
+          vv[r][e] = (T)re;
+          vv[r][e + 1] = (T)im;
+        }
+#pragma unroll
+      for (int k = 0; k < KC; ++k) {
+        Rp p[P];
+        unpack(Sp{}, raw[k], p);
+#pragma unroll
+        for (int r = 0; r < RB; ++r)
+#pragma unroll
+          for (int e = 0; e < P; e += 2) {
+            acc[k][r][0] += (T)p[e] * vv[r][e];
+            acc[k][r][0] += (T)p[e + 1] * vv[r][e + 1];
+            acc[k][r][1] += (T)p[e] * vv[r][e + 1];
+            acc[k][r][1] -= (T)p[e + 1] * vv[r][e];
+          }
+      }
+    }
+    double s[32];
+#pragma unroll
+    for (int q = 0; q < 32; ++q) s[q] = widen(acc[(q / 2) / RB][(q / 2) % RB][q & 1]);
+    const double total = warp_scatter_sum(s);
+    __syncthreads();
+    part[threadIdx.x >> 5][threadIdx.x & 31] = total;
+    __syncthreads();
+    if (threadIdx.x < 16) {
+      const int k = threadIdx.x / RB, r = threadIdx.x % RB;
+      double re = 0, im = 0;
+#pragma unroll
+      for (int w = 0; w < 8; ++w) {
+        re += part[w][2 * threadIdx.x];
+        im += part[w][2 * threadIdx.x + 1];
+      }
+      if (k < kc && r < rb) out[(b * nvec + k0 + k) * R + r0 + r] = {(Rc)re, (Rc)im};
+    }
+  }
+}
+
+// The same for 16-bit vectors and fields of one type, on the tensor cores: rows
+// are 16 subspace vectors, columns 8 right-hand sides, k the block's reals (exact
+// 16-bit products).  As in hop_tc.cuh k may be permuted: lane (g, t) loads granule
+// 4 i + t of vectors g and g + 8 and of field g, its four words are two k16 steps.
+// Re <phi, v> takes (v_re, v_im), Im (v_im, -v_re).  FP32 sums over 16 groups of
+// four granules (512 products) go to a double-float pair; the sums over warps are
+// FP64.  Reads each vector once for up to 16 right-hand sides.
+constexpr int RT_WARPS = 8, RT_FLUSH = 16;
+template <typename S, int NT>
+__global__ void __launch_bounds__(32 * RT_WARPS, 2) k_restrict_tc(const uint4* __restrict__ phi, size_t pstride,
+                                                                  int nvec, const uint4* __restrict__ v,
+                                                                  size_t vstride, int R, BlockArgs ba, float2* out) {
+  __shared__ double2 part[RT_WARPS][16][8];
+  const size_t b = blockIdx.x;
+  const int k0 = blockIdx.y * 16;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
+  const int per = ba.Ls * 3;                     // granules of a 4D site
+  const int groups = ba.spb * per / 4;
+  const uint4* p0 = phi + (size_t)min(k0 + g, nvec - 1) * pstride;
+  const uint4* p1 = phi + (size_t)min(k0 + g + 8, nvec - 1) * pstride;
+  float hi[NT][2][4], lo[NT][2][4], acc[NT][2][4];
+#pragma unroll
+  for (int n = 0; n < NT; ++n)
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) hi[n][h][i] = lo[n][h][i] = acc[n][h][i] = 0.f;
+  constexpr int U = 4;
+  int count = 0;
+  for (int i0 = w; i0 < groups; i0 += U * RT_WARPS) {
+    uint4 a0[U], a1[U], bv[U][NT];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int i = i0 + u * RT_WARPS;
+      const int gr = 4 * min(i, groups - 1) + t;
+      const size_t at = (size_t)__ldg(ba.block_sites + b * ba.spb + gr / per) * per + gr % per;
+      a0[u] = __ldg(p0 + at);
+      a1[u] = __ldg(p1 + at);
+#pragma unroll
+      for (int n = 0; n < NT; ++n)
+        bv[u][n] = (8 * n + g < R && i < groups) ? __ldg(v + (size_t)(8 * n + g) * vstride + at) : make_uint4(0u, 0u, 0u, 0u);
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+      for (int n = 0; n < NT; ++n) {
+        const uint4 x = bv[u][n];
+        // (re, im) -> (im, -re)
+        auto turn = [](unsigned z) { return __byte_perm(z, 0u, 0x1032u) ^ 0x80000000u; };
+        tch::mma<S>(acc[n][0], a0[u].x, a1[u].x, a0[u].y, a1[u].y, x.x, x.y);
+        tch::mma<S>(acc[n][0], a0[u].z, a1[u].z, a0[u].w, a1[u].w, x.z, x.w);
+        tch::mma<S>(acc[n][1], a0[u].x, a1[u].x, a0[u].y, a1[u].y, turn(x.x), turn(x.y));
+        tch::mma<S>(acc[n][1], a0[u].z, a1[u].z, a0[u].w, a1[u].w, turn(x.z), turn(x.w));
+      }
+    if ((++count) * U >= RT_FLUSH || i0 + U * RT_WARPS >= groups) {
+      count = 0;
+#pragma unroll
+      for (int n = 0; n < NT; ++n)
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            float s, e;
+            two_sum(hi[n][h][i], acc[n][h][i], s, e);
+            hi[n][h][i] = s;
+            lo[n][h][i] = __fadd_rn(lo[n][h][i], e);
+            acc[n][h][i] = 0.f;
+          }
+    }
+  }
+#pragma unroll
+  for (int n = 0; n < NT; ++n) {
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      part[w][g + 8 * (i / 2)][2 * t + (i & 1)] = make_double2(widen(hi[n][0][i]) + widen(lo[n][0][i]),
+                                                               widen(hi[n][1][i]) + widen(lo[n][1][i]));
+    __syncthreads();
+    const int k = threadIdx.x / 8, r = threadIdx.x % 8;
+    if (k < 16 && k0 + k < nvec && 8 * n + r < R) {
+      double re = 0, im = 0;
+#pragma unroll
+      for (int q = 0; q < RT_WARPS; ++q) {
+        re += part[q][k][r].x;
+        im += part[q][k][r].y;
+      }
+      out[(b * nvec + k0 + k) * R + 8 * n + r] = make_float2((float)re, (float)im);
+    }
+  }
+}
+
+// c[a][k][r] = <phi_k^a, v_r> for R fields v
+void restrict_multi(Ctx& c, const Subspace& s, const uint4* v, int vprec, int R, void* cvec, int cprec) {
+  const size_t ps = s.vec_bytes(c) / 16, vs = c.field_bytes(vprec) / 16;
   HDCG_REQUIRE((cprec == HDCG_F64) == (s.prec == HDCG_F64), HDCG_ERR_ARG,
                "coarse vectors are FP64 exactly when the subspace is FP64");
+  HDCG_REQUIRE(R >= 1 && R <= RMAX, HDCG_ERR_ARG, "1..16 right-hand sides");
+  const BlockArgs ba = block_args(c, s);
+  ++c.launches;
+  if (s.prec == HDCG_F16 && vprec == HDCG_F16) {
+    const dim3 grid((unsigned)s.Vc, (unsigned)((s.nvec + 15) / 16));
+    if (R <= 8)
+      k_restrict_tc<f16_t, 1><<<grid, 32 * RT_WARPS, 0, c.stream>>>(s.vecs.as<uint4>(), ps, s.nvec, v, vs, R, ba,
+                                                                    (float2*)cvec);
+    else
+      k_restrict_tc<f16_t, 2><<<grid, 32 * RT_WARPS, 0, c.stream>>>(s.vecs.as<uint4>(), ps, s.nvec, v, vs, R, ba,
+                                                                    (float2*)cvec);
+    HDCG_CUDA(cudaGetLastError());
+    return;
+  }
   DISPATCH_SUB(s.prec, Sp, {
     DISPATCH_PREC(vprec, Sv, {
       using Rc = typename std::conditional<std::is_same<Sp, f64_t>::value, double, float>::type;
-      k_restrict<Sp, Sv, Rc><<<(unsigned)s.Vc, 256, 0, c.stream>>>(s.vecs.as<uint4>(), pstride, s.nvec, v,
-                                                                   block_args(c, s), (typename CV<Rc>::T*)cvec);
+      using V = typename CV<Rc>::T;
+      if (R == 1)
+        k_restrict<Sp, Sv, Rc, 16, 1><<<dim3((unsigned)s.Vc, (unsigned)((s.nvec + 15) / 16)), 256, 0, c.stream>>>(
+            s.vecs.as<uint4>(), ps, s.nvec, v, vs, R, ba, (V*)cvec);
+      else
+        k_restrict<Sp, Sv, Rc, 4, 4><<<dim3((unsigned)s.Vc, (unsigned)((s.nvec + 3) / 4)), 256, 0, c.stream>>>(
+            s.vecs.as<uint4>(), ps, s.nvec, v, vs, R, ba, (V*)cvec);
     });
   });
   HDCG_CUDA(cudaGetLastError());
-  ++c.launches;
+}
+
+void restrict_field(Ctx& c, const Subspace& s, const uint4* v, int vprec, void* cvec, int cprec) {
+  restrict_multi(c, s, v, vprec, 1, cvec, cprec);
 }
 
 template <typename Sp, typename So, typename Rc>
@@ -1417,85 +1614,100 @@ void coarse_apply_noalloc(Ctx& c, const Coarse& A, const void* x64, void* y64) {
 // right-hand sides are stored [a][k][r] (right-hand side fastest).
 // ---------------------------------------------------------------------------
 
-// c[a][k][r] = <phi_k^a, v_r> for R fields v (one Gram pass reads phi once)
-void restrict_multi(Ctx& c, const Subspace& s, const uint4* v, int vprec, int R, void* cvec, int cprec) {
-  const size_t nc = s.Vc * s.nvec * (size_t)R;
-  DevMem G;
-  G.ensure(nc * sizeof(double2));
-  block_gram(c, s, v, R, vprec, c.field_bytes(vprec) / 16, G.as<double2>(), (size_t)s.nvec * R, GramPhase{});
-  cvec_convert(c, G.p, HDCG_F64, cvec, cprec, nc);
+// out_r = f_r (add_r + sum_k c[b][k][r] phi_k), RB right-hand sides per pass over
+// the vectors.  One thread per granule of the subspace: its 16 bytes of each vector
+// serve RB right-hand sides from registers, c is a broadcast from L1.  Bound by the
+// FP32 multiply-adds for RB 8 and by the stream of the vectors below.  (Staging the
+// vectors in shared memory tiles instead cost two 16-byte shared loads per 16
+// multiply-adds.)  The added field may be FP16 under an FP32 or FP64 output.
+template <typename So>
+__device__ __forceinline__ void store_complex(uint4* f, int z, size_t site5, size_t n5, typename Store<So>::real re,
+                                              typename Store<So>::real im) {
+  if constexpr (Store<So>::chunks == 6) {
+    reinterpret_cast<float2*>(f + (size_t)(z / 2) * n5 + site5)[z & 1] = make_float2(re, im);
+  } else if constexpr (Store<So>::chunks == 12) {
+    const typename Store<So>::real r[2] = {re, im};
+    f[(size_t)z * n5 + site5] = pack(So{}, r);
+  } else {
+    typename Store<So>::real r[8] = {re, im, 0, 0, 0, 0, 0, 0};
+    reinterpret_cast<unsigned*>(f)[site5 * 12 + 4 * (z % 3) + z / 3] = pack(So{}, r).x;
+  }
 }
 
-// out_r = f_r (add_r + sum_k c[b][k][r] phi_k)  (tile of all vectors in shared memory);
-// the added field may be stored in a narrower precision Sa than the output
-template <typename Sp, typename So, typename Rt, typename Sa>
-__global__ void __launch_bounds__(256) k_prolong_multi(const uint4* phi, size_t pstride, int n, BlockArgs ba,
+template <typename Sp, typename So, typename Rt, typename Sa, int RB>
+__global__ void __launch_bounds__(256) k_prolong_multi(const uint4* __restrict__ phi, size_t pstride, int n,
+                                                       const int* __restrict__ bos, size_t n5, int lslog2,
                                                        const typename CV<Rt>::T* __restrict__ cv, int R,
                                                        uint4* out, const uint4* add, size_t ostride, size_t astride,
                                                        const double* un_num, const double* un_den) {
+  using Rp = typename Store<Sp>::real;
   using Ro = typename Store<So>::real;
   using Ra = typename Store<Sa>::real;
-  constexpr int C = Store<So>::chunks, P = Store<So>::per_chunk;
-  extern __shared__ __align__(16) unsigned char smraw[];
-  Rt* xs = reinterpret_cast<Rt*>(smraw);
-  Rt* cs = xs + (size_t)n * TROW;    // [k][r] complex
+  constexpr int C = Store<Sp>::chunks, P = Store<Sp>::per_chunk;
   __shared__ Rt unscale[RMAX];
-  const size_t b = blockIdx.x;
-  for (int q = threadIdx.x; q < n * R; q += blockDim.x) {
-    const typename CV<Rt>::T v = cv[b * n * R + q];
-    cs[2 * q] = v.x;
-    cs[2 * q + 1] = v.y;
-  }
   if (threadIdx.x < RMAX)
     unscale[threadIdx.x] = (un_num && (int)threadIdx.x < R) ? (Rt)sqrt(un_den[threadIdx.x] / un_num[0]) : Rt(1);
-  const int nsites = ba.spb * ba.Ls;
-  const int units = R * TILE * C;
-  for (int tile0 = 0; tile0 < nsites; tile0 += TILE) {
-    __syncthreads();
-    load_tile<Sp, Rt>(xs, phi, pstride, n, ba, b, tile0);
-    __syncthreads();
-    for (int u = threadIdx.x; u < units; u += blockDim.x) {
-      const int t = u % TILE;
-      const int ch = (u / TILE) % C;
-      const int r = u / (C * TILE);
-      Rt o[P];
+  __syncthreads();
+  const size_t i = (size_t)blockIdx.x * 256 + threadIdx.x;
+  if (i >= n5 * C) return;
+  const int ch = C == 3 ? (int)(i % 3) : (int)(i / n5);
+  const size_t site5 = C == 3 ? i / 3 : i % n5;
+  const int r0 = blockIdx.y * RB, rb = min(RB, R - r0);
+  const size_t b = (size_t)__ldg(bos + (site5 >> lslog2));
+  const typename CV<Rt>::T* cb = cv + b * n * R + r0;
+  const uint4* pk = phi + granule_at<Sp>(ch, site5, n5);
+  Rt acc[RB][P];
 #pragma unroll
-      for (int i = 0; i < P; ++i) o[i] = 0;
-      for (int k = 0; k < n; ++k) {
-        const Rt cr = cs[2 * (k * R + r)], ci = cs[2 * (k * R + r) + 1];
-        const Rt* xr = xs + k * TROW + t * 24;
+  for (int r = 0; r < RB; ++r)
 #pragma unroll
-        for (int i = 0; i < P; i += 2) {
-          const Rt xre = xr[real_of<So>(ch, i)], xim = xr[real_of<So>(ch, i) + 1];
-          o[i] += cr * xre - ci * xim;
-          o[i + 1] += cr * xim + ci * xre;
-        }
-      }
-      const size_t site5 = block_site5(ba, b, tile0 + t);
-      if (add) {
-        if constexpr (std::is_same<So, Sa>::value) {
-          Ra av[P];
-          unpack(Sa{}, __ldg(add + r * astride + granule_at<Sa>(ch, site5, ba.n5)), av);
+    for (int e = 0; e < P; ++e) acc[r][e] = 0;
+  for (int k = 0; k < n; k += 4) {
+    uint4 raw[4];
 #pragma unroll
-          for (int i = 0; i < P; ++i) o[i] += (Rt)av[i];
-        } else {
-          // FP16 added to FP32 or FP64: one 32-bit word (spin, colour) per complex number
-          static_assert(std::is_same<Sa, f16_t>::value && Store<So>::chunks != 3, "the added field is FP16");
-          const unsigned* words = reinterpret_cast<const unsigned*>(add + r * astride) + site5 * 12;
+    for (int u = 0; u < 4; ++u) raw[u] = __ldg(pk + (size_t)min(k + u, n - 1) * pstride);
 #pragma unroll
-          for (int i = 0; i < P; i += 2) {
-            const int z = (ch * P + i) / 2;                      // spin * 3 + colour
-            const float2 av = h2f(__ldg(words + 4 * (z % 3) + z / 3));
-            o[i] += (Rt)av.x;
-            o[i + 1] += (Rt)av.y;
+    for (int u = 0; u < 4; ++u) {
+      if (k + u < n) {
+        Rp p[P];
+        unpack(Sp{}, raw[u], p);
+#pragma unroll
+        for (int r = 0; r < RB; ++r) {
+          const typename CV<Rt>::T q = cb[(size_t)(k + u) * R + min(r, rb - 1)];
+#pragma unroll
+          for (int e = 0; e < P; e += 2) {
+            acc[r][e] += q.x * (Rt)p[e];
+            acc[r][e] -= q.y * (Rt)p[e + 1];
+            acc[r][e + 1] += q.x * (Rt)p[e + 1];
+            acc[r][e + 1] += q.y * (Rt)p[e];
           }
         }
       }
-      const Rt f = unscale[r];
-      Ro w[P];
+    }
+  }
 #pragma unroll
-      for (int i = 0; i < P; ++i) w[i] = (Ro)(f * o[i]);
-      out[r * ostride + granule_at<So>(ch, site5, ba.n5)] = pack(So{}, w);
+  for (int r = 0; r < RB; ++r) {
+    if (r >= rb) break;
+    const Rt f = unscale[r0 + r];
+#pragma unroll
+    for (int e = 0; e < P; e += 2) {
+      const int z = real_of<Sp>(ch, e) / 2;
+      Rt re = acc[r][e], im = acc[r][e + 1];
+      if (add) {
+        Ra ar, ai;
+        load_complex<Sa>(add + (r0 + r) * astride, z, site5, n5, ar, ai);
+        re += (Rt)ar;
+        im += (Rt)ai;
+      }
+      acc[r][e] = f * re;
+      acc[r][e + 1] = f * im;
+      if constexpr (Store<So>::chunks != C)
+        store_complex<So>(out + (r0 + r) * ostride, z, site5, n5, (Ro)acc[r][e], (Ro)acc[r][e + 1]);
+    }
+    if constexpr (Store<So>::chunks == C) {
+      Ro o[P];
+#pragma unroll
+      for (int e = 0; e < P; ++e) o[e] = (Ro)acc[r][e];
+      out[(r0 + r) * ostride + granule_at<So>(ch, site5, n5)] = pack(So{}, o);
     }
   }
 }
@@ -1503,13 +1715,16 @@ __global__ void __launch_bounds__(256) k_prolong_multi(const uint4* phi, size_t 
 template <typename Sp, typename So, typename Rt, typename Sa>
 static void launch_prolong_multi(Ctx& c, const Subspace& s, const void* cvec, int R, uint4* out, const uint4* add,
                                  size_t ostride, size_t astride, const double* un_num, const double* un_den) {
-  const int n = s.nvec;
-  const size_t sm = tile_smem<Rt>(n) + (size_t)n * R * 2 * sizeof(Rt);
-  auto fn = k_prolong_multi<Sp, So, Rt, Sa>;
-  set_smem_limit((const void*)fn, sm);
-  fn<<<(unsigned)s.Vc, 256, sm, c.stream>>>(s.vecs.as<uint4>(), s.vec_bytes(c) / 16, n, block_args(c, s),
-                                             (const typename CV<Rt>::T*)cvec, R, out, add, ostride, astride, un_num,
-                                             un_den);
+  const unsigned gx = (unsigned)((c.n5 * Store<Sp>::chunks + 255) / 256);
+  auto go = [&](auto fn, int rb) {
+    fn<<<dim3(gx, (unsigned)((R + rb - 1) / rb)), 256, 0, c.stream>>>(
+        s.vecs.as<uint4>(), s.vec_bytes(c) / 16, s.nvec, s.block_of_site.as<int>(), c.n5, c.lslog2,
+        (const typename CV<Rt>::T*)cvec, R, out, add, ostride, astride, un_num, un_den);
+  };
+  // right-hand sides per pass: as many as there are, up to 8 (64 sums per thread)
+  if (R <= 2) go(k_prolong_multi<Sp, So, Rt, Sa, 2>, 2);
+  else if (R <= 4) go(k_prolong_multi<Sp, So, Rt, Sa, 4>, 4);
+  else go(k_prolong_multi<Sp, So, Rt, Sa, 8>, 8);
 }
 
 void prolong_multi(Ctx& c, const Subspace& s, const void* cvec, int cprec, int R, uint4* out, int oprec,

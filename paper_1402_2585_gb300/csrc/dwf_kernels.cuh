@@ -8,6 +8,7 @@
 #include "common.cuh"
 #include "context.h"
 #include "dfloat.cuh"
+#include "mma.cuh"
 
 namespace hdcg {
 
