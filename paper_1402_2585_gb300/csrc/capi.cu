@@ -393,7 +393,7 @@ int hdcg_restrict(hdcg_t h, const void* v, int prec, void* cv) {
     const size_t nc = c.sub->Vc * c.sub->nvec;
     c.canon_in.ensure(c.field_bytes(prec));
     canon_to_internal(c, v, prec, c.canon_in.as<uint4>(), prec);
-    DevMem tmp;
+    DevMem& tmp = c.coarse_io[0];
     tmp.ensure(nc * 16);
     restrict_field(c, *c.sub, c.canon_in.as<uint4>(), prec, tmp.p, cp);
     cvec_convert(c, tmp.p, cp, cv, HDCG_F64, nc);
@@ -410,7 +410,7 @@ int hdcg_prolong(hdcg_t h, const void* cv, void* v, int prec) {
     HDCG_REQUIRE(c.sub, HDCG_ERR_STATE, "no subspace");
     const int cp = c.sub->prec == HDCG_F64 ? HDCG_F64 : HDCG_F32;
     const size_t nc = c.sub->Vc * c.sub->nvec;
-    DevMem tmp;
+    DevMem& tmp = c.coarse_io[0];
     tmp.ensure(nc * 16);
     cvec_convert(c, cv, HDCG_F64, tmp.p, cp, nc);
     c.canon_out.ensure(c.field_bytes(prec));
@@ -428,7 +428,7 @@ int hdcg_coarse_apply(hdcg_t h, const void* x, void* y) {
     HDCG_REQUIRE(c.coarse, HDCG_ERR_STATE, "no coarse operator");
     const int cp = c.coarse->vec_prec();
     const size_t nc = c.coarse->Vc * c.coarse->nvec;
-    DevMem tmp;
+    DevMem& tmp = c.coarse_io[0];
     tmp.ensure(2 * nc * 16);
     char* xi = tmp.as<char>();
     char* yi = xi + nc * 16;

@@ -1218,7 +1218,7 @@ template <typename AT, typename R>
 static void coarse_apply_t(Ctx& c, const Coarse& A, const void* x, void* y, double* xAx) {
   using V = typename CV<R>::T;
   const size_t nc = A.Vc * A.nvec;
-  DevMem part;
+  DevMem& part = c.coarse_io[1];
   part.ensure(CGROUPS * nc * sizeof(V));
   const unsigned g = (unsigned)(A.Vc * CGROUPS);
   Reduction red{};
@@ -2082,7 +2082,7 @@ template <typename AT, typename R_>
 static void coarse_apply_multi_t(Ctx& c, const Coarse& A, int R, const void* x, void* y) {
   using V = typename CV<R_>::T;
   const size_t nc = A.Vc * A.nvec * (size_t)R;
-  DevMem tmp;
+  DevMem& tmp = c.coarse_io[1];
   tmp.ensure((2 + CGROUPS) * nc * sizeof(V));
   V* xi = tmp.as<V>();
   V* yi = xi + nc;

@@ -221,6 +221,52 @@ __global__ void k_x_to_tc(const float2* __restrict__ x, uint4* __restrict__ xtc,
   }
 }
 
+// The same from canonical vectors [r][a][k] (complex double): consecutive threads
+// take consecutive k groups of a right-hand side, 128 contiguous bytes each.
+__global__ void k_canon_to_tc(const double2* __restrict__ x, uint4* __restrict__ xtc, size_t Vc, int n, int R, int Rp,
+                              int Kp, const unsigned* __restrict__ xmax) {
+  const int KG = Kp / 8;
+  const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= Vc * KG * Rp) return;
+  const int kg = (int)(t % KG);
+  const size_t a = (t / KG) % Vc;
+  const int r = (int)(t / ((size_t)KG * Vc));
+  const float s = r < R ? pow2f(scale_exp(xmax[r])) : 0.f;
+  __align__(16) __half v[4][8];
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    const int k = kg * 8 + q;
+    double2 xv = make_double2(0., 0.);
+    if (r < R && k < n) xv = x[((size_t)r * Vc + a) * n + k];
+    const float re = (float)xv.x * s, im = (float)xv.y * s;
+    const __half rh = __float2half_rn(re), ih = __float2half_rn(im);
+    v[0][q] = rh;
+    v[1][q] = ih;
+    v[2][q] = __float2half_rn(re - __half2float(rh));
+    v[3][q] = __float2half_rn(im - __half2float(ih));
+  }
+  char* tile = reinterpret_cast<char*>(xtc) + a * (size_t)(4 * Rp) * Kp * 2;
+#pragma unroll
+  for (int part = 0; part < 4; ++part) {
+    const int c = 4 * r + part;
+    *reinterpret_cast<uint4*>(tile + (size_t)(c / 8) * (Kp * 16) + kg * 128 + (c % 8) * 16) =
+        *reinterpret_cast<const uint4*>(v[part]);
+  }
+}
+
+// xmax[r] of canonical vectors (grid y: right-hand side)
+__global__ void k_canon_max(const double2* __restrict__ x, size_t ne, unsigned* xmax) {
+  const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  float m = 0.f;
+  if (t < ne) {
+    const double2 v = x[blockIdx.y * ne + t];
+    m = fmaxf(fabsf((float)v.x), fabsf((float)v.y));
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(FULL_MASK, m, o));
+  if ((threadIdx.x & 31) == 0 && m > 0.f) atomicMax(xmax + blockIdx.y, __float_as_uint(m));
+}
+
 // per-right-hand-side max(|Re x|, |Im x|) as float bits (atomicMax on non-negative floats)
 __global__ void k_cmax(const float2* __restrict__ x, size_t ne, int R, unsigned* xmax) {
   const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -251,6 +297,7 @@ struct TcArgs {
   const unsigned* xmax;
   const float2* x;     // FP32 X for <X, Y> (nullable)
   float2* y;
+  double2* y64;        // not null: Y canonical, [r][site][j] complex double, instead of y
   const int* skip;     // nonzero: the launch has nothing to do (nullable)
   unsigned* err;       // bit flags of expired waits
   int Vc, n, R, sites, MS, Kp, NS, stages, ncols;
@@ -426,6 +473,10 @@ __global__ void __launch_bounds__(TC_THREADS, 2) k_capply_tc(TcArgs g, Reduction
           const float t = __shfl_xor_sync(FULL_MASK, Q, 1);
           float v = (ri ? t + P : P - t) * (inv[r] * sinv);
           if (valid) {
+            if (g.y64) {   // lanes run over (j, ri): 256 contiguous bytes per right-hand side
+              reinterpret_cast<double*>(g.y64)[2 * (((size_t)r * g.Vc + site) * g.n + j) + ri] = (double)v;
+              continue;
+            }
             const size_t e = ((size_t)site * g.n + j) * g.R + r;
             if (g.x) {
               const float xv = reinterpret_cast<const float*>(g.x)[2 * e + ri];
@@ -515,7 +566,7 @@ void coarse_tc_to_b(Ctx& c, Coarse& A, int R, const float2* x, const unsigned* x
 
 // one launch with cpsm (1 or 2) persistent CTAs per SM and the matching ring
 static void launch_tc(Ctx& c, Coarse& A, int R, const float2* x, float2* y, const unsigned* xmax, const int* skip,
-                      double* dot_result, double shift, int cpsm) {
+                      double* dot_result, double shift, int cpsm, double2* y64) {
   const TcGeom g = tc_geom(A.nvec, R, tc_parts(A), cpsm == 1 ? TC_RING_BYTES_1 : TC_RING_BYTES);
   TcArgs a;
   a.Atc = A.Atc.as<uint4>();
@@ -524,6 +575,7 @@ static void launch_tc(Ctx& c, Coarse& A, int R, const float2* x, float2* y, cons
   a.xmax = xmax;
   a.x = x;
   a.y = y;
+  a.y64 = y64;
   a.skip = skip;
   a.err = &A.tcs.as<TcState>()->err;
   a.Vc = (int)A.Vc;
@@ -564,8 +616,8 @@ static void launch_tc(Ctx& c, Coarse& A, int R, const float2* x, float2* y, cons
 // the stages in flight), and keeps the faster.  Both run the same MMAs in the
 // same order, so the choice never changes a result.  Inside a stream capture
 // the two-CTA shape runs untimed.
-void coarse_tc_apply(Ctx& c, Coarse& A, int R, const float2* x, float2* y, const unsigned* xmax, const int* skip,
-                     double* dot_result, double shift) {
+static void tc_apply(Ctx& c, Coarse& A, int R, const float2* x, float2* y, const unsigned* xmax, const int* skip,
+                     double* dot_result, double shift, double2* y64) {
   int cfg = c.tc_force ? c.tc_force : A.tc_cfg[R];
   if (cfg == 0) {
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
@@ -578,9 +630,9 @@ void coarse_tc_apply(Ctx& c, Coarse& A, int R, const float2* x, float2* y, const
       HDCG_CUDA(cudaEventCreate(&e1));
       float best = 1e30f;
       for (int cand : {2, 1}) {
-        launch_tc(c, A, R, x, y, xmax, skip, dot_result, shift, cand);
+        launch_tc(c, A, R, x, y, xmax, skip, dot_result, shift, cand, y64);
         HDCG_CUDA(cudaEventRecord(e0, c.stream));
-        for (int i = 0; i < 3; ++i) launch_tc(c, A, R, x, y, xmax, skip, dot_result, shift, cand);
+        for (int i = 0; i < 3; ++i) launch_tc(c, A, R, x, y, xmax, skip, dot_result, shift, cand, y64);
         HDCG_CUDA(cudaEventRecord(e1, c.stream));
         HDCG_CUDA(cudaEventSynchronize(e1));
         float ms = 0.f;
@@ -595,7 +647,11 @@ void coarse_tc_apply(Ctx& c, Coarse& A, int R, const float2* x, float2* y, const
       A.tc_cfg[R] = cfg;
     }
   }
-  launch_tc(c, A, R, x, y, xmax, skip, dot_result, shift, cfg);
+  launch_tc(c, A, R, x, y, xmax, skip, dot_result, shift, cfg, y64);
+}
+void coarse_tc_apply(Ctx& c, Coarse& A, int R, const float2* x, float2* y, const unsigned* xmax, const int* skip,
+                     double* dot_result, double shift) {
+  tc_apply(c, A, R, x, y, xmax, skip, dot_result, shift, nullptr);
 }
 
 // ---------------------------------------------------------------------------------
@@ -836,7 +892,7 @@ int coarse_solve_canon(Ctx& c, Coarse& A, int R, const void* b64, void* x64, dou
   HDCG_REQUIRE(R >= 1 && R <= RMAX, HDCG_ERR_ARG, "1..16 right-hand sides");
   const size_t ne = A.Vc * A.nvec, nc = ne * R;
   const unsigned gt = (unsigned)((nc + 255) / 256);
-  DevMem tmp;
+  DevMem& tmp = c.coarse_io[0];
   int it;
   if (A.l2) A.l2->last_broke = 0;
   if (A.vec_prec() == HDCG_F32) {
@@ -899,24 +955,25 @@ void coarse_apply_multi_canon(Ctx& c, Coarse& A, int R, const void* x64, void* y
   const size_t ne = A.Vc * A.nvec, nc = ne * R;
   const unsigned gt = (unsigned)((nc + 255) / 256);
   if (coarse_tc_supported(A)) {
+    // the operand straight from x, the result straight into y: no staging
     coarse_tc_prepare(c, A);
-    DevMem tmp;
-    tmp.ensure(2 * nc * sizeof(float2));
-    float2* xi = tmp.as<float2>();
-    float2* yi = xi + nc;
-    k_canon_to_multi<float2><<<gt, 256, 0, c.stream>>>((const double2*)x64, xi, ne, R);
+    const double2* x = (const double2*)x64;
     unsigned* xmax = A.tcs.as<TcState>()->xmax;
-    coarse_tc_max(c, xi, ne, R, xmax);
-    coarse_tc_to_b(c, A, R, xi, xmax, nullptr);
-    coarse_tc_apply(c, A, R, xi, yi, xmax, nullptr, nullptr, 0.0);
-    k_multi_to_canon<float2><<<gt, 256, 0, c.stream>>>(yi, (double2*)y64, ne, R);
-    c.launches += 2;
+    HDCG_CUDA(cudaMemsetAsync(xmax, 0, RMAX * sizeof(unsigned), c.stream));
+    k_canon_max<<<dim3((unsigned)((ne + 255) / 256), (unsigned)R), 256, 0, c.stream>>>(x, ne, xmax);
+    const TcGeom g = tc_geom(A.nvec, R, tc_parts(A));
+    A.xtc.ensure(A.Vc * (size_t)g.b_bytes);
+    const size_t nt = A.Vc * (size_t)(g.Kp / 8) * g.Rp;
+    k_canon_to_tc<<<(unsigned)((nt + 255) / 256), 256, 0, c.stream>>>(x, A.xtc.as<uint4>(), A.Vc, A.nvec, R, g.Rp,
+                                                                      g.Kp, xmax);
     HDCG_CUDA(cudaGetLastError());
+    c.launches += 2;
+    tc_apply(c, A, R, nullptr, nullptr, xmax, nullptr, nullptr, 0.0, (double2*)y64);
     coarse_tc_check(c, A);
     return;
   }
   // FP32 / FP64 operator: the CUDA-core kernel on [a][k][r] complex double
-  DevMem tmp;
+  DevMem& tmp = c.coarse_io[0];
   tmp.ensure(2 * nc * sizeof(double2));
   double2* xi = tmp.as<double2>();
   double2* yi = xi + nc;

@@ -135,6 +135,11 @@ struct Ctx {
   int tc_force = 0;              // 1, 2: the tensor-core stencil's CTAs per SM (hdcg_set_coarse_tc_shape)
   DevMem red_partials, red_ticket, scalars;
   DevMem canon_in, canon_out;  // canonical <-> internal staging
+  // coarse vectors of the calls on canonical coarse vectors: kept by the handle
+  // (cudaMalloc and cudaFree cost more than a small coarse apply), two because a
+  // call's own staging and the partial products of the apply inside it are alive
+  // together; every call synchronises before it returns
+  mutable DevMem coarse_io[2];
 
   Subspace* sub = nullptr;
   Coarse* coarse = nullptr;

@@ -1058,7 +1058,7 @@ void level2_restrict_canon(Ctx& c, const Coarse& A, int R, const void* x64, void
   HDCG_REQUIRE(R >= 1 && R <= RMAX, HDCG_ERR_ARG, "1..16 right-hand sides");
   const Level2& L = *A.l2;
   const size_t ne = L.Vc1 * L.n1, n2 = L.Vc2 * L.nvec;
-  DevMem x, cc;
+  DevMem &x = c.coarse_io[0], &cc = c.coarse_io[1];
   x.ensure(ne * R * sizeof(float2));
   cc.ensure(n2 * R * sizeof(float2));
   coarse_canon_to_multi(c, x64, x.as<float2>(), ne, R);
@@ -1073,7 +1073,7 @@ void level2_prolong_canon(Ctx& c, const Coarse& A, int R, const void* c64, void*
   HDCG_REQUIRE(R >= 1 && R <= RMAX, HDCG_ERR_ARG, "1..16 right-hand sides");
   const Level2& L = *A.l2;
   const size_t ne = L.Vc1 * L.n1, n2 = L.Vc2 * L.nvec;
-  DevMem x, cc;
+  DevMem &x = c.coarse_io[0], &cc = c.coarse_io[1];
   x.ensure(ne * R * sizeof(float2));
   cc.ensure(n2 * R * sizeof(float2));
   coarse_canon_to_multi(c, c64, cc.as<float2>(), n2, R);

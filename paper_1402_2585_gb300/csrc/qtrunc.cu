@@ -414,7 +414,7 @@ void qtrunc_precondition_canon(Ctx& c, Coarse& A, int R, const void* x64, void* 
   HDCG_REQUIRE(A.qt.order > 0, HDCG_ERR_STATE, "no coarse preconditioner");
   HDCG_REQUIRE(R >= 1 && R <= RMAX, HDCG_ERR_ARG, "1..16 right-hand sides");
   const size_t ne = A.Vc * A.nvec;
-  DevMem x, y;
+  DevMem &x = c.coarse_io[0], &y = c.coarse_io[1];
   x.ensure(ne * R * sizeof(float2));
   y.ensure(ne * R * sizeof(float2));
   coarse_canon_to_multi(c, x64, x.as<float2>(), ne, R);
