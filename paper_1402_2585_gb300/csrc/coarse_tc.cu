@@ -305,7 +305,13 @@ struct TcArgs {
   float shift;         // Y = (A + shift) X (needs x)
   int parts;           // 1: FP16 operator, 2: FP32 operator as FP16 hi + lo
   const int* sexp;     // per-site scale exponents of the tiled operator
+  // The 81 couplings of a pair split over nsplit work items (items of one pair add
+  // up: part s goes to y + s part; the shift joins part 0).  1 for operators with
+  // enough pairs to fill the chip.
+  int nsplit;
+  size_t part;
 };
+__device__ __forceinline__ int split_begin(int s, int nsplit) { return s * 81 / nsplit; }
 
 __global__ void __launch_bounds__(TC_THREADS, 2) k_capply_tc(TcArgs g, Reduction red) {
   extern __shared__ __align__(128) unsigned char smem[];
@@ -342,7 +348,7 @@ __global__ void __launch_bounds__(TC_THREADS, 2) k_capply_tc(TcArgs g, Reduction
   __syncthreads();
   tc::fence_after_sync();
   const uint32_t tmem = *tslot;
-  const int npairs = (g.Vc + g.sites - 1) / g.sites;
+  const int items = (g.Vc + g.sites - 1) / g.sites * g.nsplit;   // (pair, part), part fastest
   double dot[RMAX];
 #pragma unroll
   for (int r = 0; r < RMAX; ++r) dot[r] = 0.0;
@@ -355,14 +361,15 @@ __global__ void __launch_bounds__(TC_THREADS, 2) k_capply_tc(TcArgs g, Reduction
     __shared__ int snb[2 * 81];
     uint32_t it = 0;
     bool ok = true;
-    for (int p = blockIdx.x; ok && p < npairs; p += gridDim.x) {
-      const int s0 = p * g.sites;
+    for (int p = blockIdx.x; ok && p < items; p += gridDim.x) {
+      const int s0 = p / g.nsplit * g.sites;
+      const int l0 = split_begin(p % g.nsplit, g.nsplit), l1 = split_begin(p % g.nsplit + 1, g.nsplit);
       const int s1 = min(s0 + 1, g.Vc - 1);
       for (int q = lane; q < g.sites * 81; q += 32)
         snb[q] = __ldg(g.cnbr + (size_t)(q < 81 ? s0 : s1) * 81 + q % 81);
       __syncwarp();
       if (lane == 0) {
-        for (int l = 0; l < 81; ++l, ++it) {
+        for (int l = l0; l < l1; ++l, ++it) {
           const int s = (int)(it % (uint32_t)g.stages);
           const uint32_t ph = (it / (uint32_t)g.stages) & 1u;
           if (!tc::mbar_wait(TC_EMPTY(s), ph ^ 1u)) {
@@ -403,14 +410,15 @@ __global__ void __launch_bounds__(TC_THREADS, 2) k_capply_tc(TcArgs g, Reduction
       int np = 0;
       bool ok = true;
       const uint32_t sbo = (uint32_t)g.Kp * 16u;
-      for (int p = blockIdx.x; ok && p < npairs; p += gridDim.x, ++np) {
+      for (int p = blockIdx.x; ok && p < items; p += gridDim.x, ++np) {
+        const int l0 = split_begin(p % g.nsplit, g.nsplit), l1 = split_begin(p % g.nsplit + 1, g.nsplit);
         if (np > 0 && !tc::mbar_wait(ACC_EMPTY, (uint32_t)(np - 1) & 1u)) {
           ok = false;
           atomicOr(g.err, 4u);
           break;
         }
         tc::fence_after_sync();
-        for (int l = 0; l < 81; ++l, ++it) {
+        for (int l = l0; l < l1; ++l, ++it) {
           const int s = (int)(it % (uint32_t)g.stages);
           const uint32_t ph = (it / (uint32_t)g.stages) & 1u;
           if (!tc::mbar_wait(TC_FULL(s), ph)) {
@@ -426,7 +434,7 @@ __global__ void __launch_bounds__(TC_THREADS, 2) k_capply_tc(TcArgs g, Reduction
             for (int p = 0; p < g.parts; ++p) {
               const uint64_t ad =
                   tc::smem_desc(abase + p * g.sites * g.a_sbytes + 2u * g.lbo_a * ks, g.lbo_a, g.sbo_a);
-              tc::mma_f16(tmem, ad, bd, g.idesc, (l | ks | p) != 0 ? 1u : 0u);
+              tc::mma_f16(tmem, ad, bd, g.idesc, (l != l0 || (ks | p) != 0) ? 1u : 0u);
             }
           }
           tc::mma_commit(TC_EMPTY(s));
@@ -448,7 +456,7 @@ __global__ void __launch_bounds__(TC_THREADS, 2) k_capply_tc(TcArgs g, Reduction
 #pragma unroll
     for (int r = 0; r < RMAX; ++r) inv[r] = r < g.R ? pow2f(-scale_exp(g.xmax[r])) : 0.f;
     int np = 0;
-    for (int p = blockIdx.x; p < npairs; p += gridDim.x, ++np) {
+    for (int p = blockIdx.x; p < items; p += gridDim.x, ++np) {
       const bool ok = tc::mbar_wait(ACC_FULL, (uint32_t)np & 1u);
       if (!__all_sync(FULL_MASK, ok)) {
         if (lane == 0) atomicOr(g.err, 32u);
@@ -462,7 +470,7 @@ __global__ void __launch_bounds__(TC_THREADS, 2) k_capply_tc(TcArgs g, Reduction
       tc::fence_before_sync();
       __syncwarp();
       if (lane == 0) tc::mbar_arrive(ACC_EMPTY);
-      const int site = p * g.sites + si;
+      const int part = p % g.nsplit, site = p / g.nsplit * g.sites + si;
       const bool valid = site < g.Vc && j < g.n;
       const float sinv = valid ? pow2f(-__ldg(g.sexp + site)) : 0.f;
 #pragma unroll
@@ -480,10 +488,10 @@ __global__ void __launch_bounds__(TC_THREADS, 2) k_capply_tc(TcArgs g, Reduction
             const size_t e = ((size_t)site * g.n + j) * g.R + r;
             if (g.x) {
               const float xv = reinterpret_cast<const float*>(g.x)[2 * e + ri];
-              v += g.shift * xv;
+              if (part == 0) v += g.shift * xv;
               dot[r] += (double)xv * (double)v;
             }
-            reinterpret_cast<float*>(g.y)[2 * e + ri] = v;
+            reinterpret_cast<float*>(g.y + part * g.part)[2 * e + ri] = v;
           }
         }
       }
@@ -566,7 +574,7 @@ void coarse_tc_to_b(Ctx& c, Coarse& A, int R, const float2* x, const unsigned* x
 
 // one launch with cpsm (1 or 2) persistent CTAs per SM and the matching ring
 static void launch_tc(Ctx& c, Coarse& A, int R, const float2* x, float2* y, const unsigned* xmax, const int* skip,
-                      double* dot_result, double shift, int cpsm, double2* y64) {
+                      double* dot_result, double shift, int cpsm, double2* y64, int nsplit = 1) {
   const TcGeom g = tc_geom(A.nvec, R, tc_parts(A), cpsm == 1 ? TC_RING_BYTES_1 : TC_RING_BYTES);
   TcArgs a;
   a.Atc = A.Atc.as<uint4>();
@@ -596,6 +604,8 @@ static void launch_tc(Ctx& c, Coarse& A, int R, const float2* x, float2* y, cons
   a.idesc = tc::idesc_f16_f32(128, g.NMMA);
   a.shift = (float)shift;
   a.parts = g.parts;
+  a.nsplit = nsplit;
+  a.part = A.Vc * A.nvec * (size_t)R;
   a.sexp = A.sexp.as<int>();
   const size_t smem = (size_t)g.stages * g.stage_bytes + (2 * g.stages + 3) * 8 + 16;
   static size_t smem_set = 0;
@@ -604,7 +614,7 @@ static void launch_tc(Ctx& c, Coarse& A, int R, const float2* x, float2* y, cons
     smem_set = std::max<size_t>(smem, 100 * 1024);
   }
   const int npairs = (int)((A.Vc + g.sites - 1) / g.sites);
-  const unsigned grid = (unsigned)std::min(npairs, cpsm * device_sms());
+  const unsigned grid = (unsigned)std::min(npairs * nsplit, cpsm * device_sms());
   const Reduction red = dot_result ? make_reduction(c, grid, RMAX, dot_result, 0) : Reduction{};
   k_capply_tc<<<grid, TC_THREADS, smem, c.stream>>>(a, red);
   HDCG_CUDA(cudaGetLastError());
@@ -795,16 +805,195 @@ __global__ void k_cgt_check(CCtlT* ctl, int R, int par, int maxiter) {
   ctl->all_done = all;
 }
 
+// ---------------------------------------------------------------------------------
+// Small coarse grids: everything of a CG iteration but the stencil in one launch.
+// The vectors of a 4^4 coarse grid (24 vectors, 4 right-hand sides: 196 KB) are a
+// few microseconds of work, but the update, the new direction, its largest entry,
+// the operand and the bookkeeping need each other's results over the whole grid:
+// as four launches of 16 to 24 CTAs they took 33 us of an iteration, k_cgt_update
+// 18 of them.  One cluster of eight CTAs meets at two cluster barriers instead.
+// With the split couplings (78 us a product on 128 of 152 SMs before, for 95 MB)
+// the batched solve of four sources on 16^4 x 16 went from 217 to 202 ms.
+// A thread owns the same (site, eight coefficients, right-hand side) items in every
+// phase.  |r|^2 sums by TwoProd and TwoSum (about 48 bits), CTAs in FP64.
+// ---------------------------------------------------------------------------------
+constexpr int CS_CTAS = 8, CS_THREADS = 512, CS_ITEMS = 4;   // at most CS_ITEMS items a thread
+struct CgStepScratch {
+  double rr[CS_CTAS][RMAX];
+  unsigned xm[CS_CTAS][RMAX];
+};
+
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+__global__ void __cluster_dims__(CS_CTAS, 1, 1) __launch_bounds__(CS_THREADS)
+    k_cgt_step(float2* x, float2* r, float2* p, const float2* w, int nsplit, size_t part, int Vc, int n, int R, int Rp,
+               int Kp, char* xtc, CCtlT* ctl, CgStepScratch* sc, int par, int maxiter, unsigned* xmax) {
+  if (ctl->all_done) return;   // written by CTA 0 behind the last barrier only
+  __shared__ float shi[CS_THREADS], slo[CS_THREADS];
+  __shared__ unsigned sxm[RMAX];
+  const int cta = blockIdx.x, tid = threadIdx.x, gid = cta * CS_THREADS + tid;
+  const int stride = CS_CTAS * CS_THREADS / Rp * Rp;    // whole groups of Rp: a thread keeps its right-hand side
+  const int q = gid % Rp, KG = Kp / 8, N = Vc * KG * Rp;
+  const bool live = gid < stride && q < R;
+  const bool run = live && !ctl->done[q];
+  if (tid < RMAX) sxm[tid] = 0u;
+  const double ro = live ? ctl->rr[par][q] : 0.0;
+  // x += alpha p, r -= alpha w, |r|^2
+  float s = 0.f, e = 0.f;
+  if (live) {
+    const double pap = ctl->pAp[q];
+    const float al = (float)(pap > 0 ? ro / pap : 0.0);
+    for (int j = gid; j < N; j += stride) {
+      const int it = j / Rp, a = it / KG, k0 = 8 * (it % KG);
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        if (k0 + k >= n) break;
+        const size_t o = ((size_t)a * n + k0 + k) * R + q;
+        float2 rv = r[o];
+        if (run) {
+          const float2 pv = p[o];
+          float2 wv = w[o], xv = x[o];
+          for (int t = 1; t < nsplit; ++t) {
+            const float2 u = w[t * part + o];
+            wv.x += u.x;
+            wv.y += u.y;
+          }
+          xv.x += al * pv.x;
+          xv.y += al * pv.y;
+          rv.x -= al * wv.x;
+          rv.y -= al * wv.y;
+          x[o] = xv;
+          r[o] = rv;
+        }
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+          const float v = c ? rv.y : rv.x, sq = __fmul_rn(v, v), d = __fmaf_rn(v, v, -sq);
+          float u;
+          two_sum(s, sq, s, u);
+          e = __fadd_rn(e, __fadd_rn(u, d));
+        }
+      }
+    }
+  }
+  shi[tid] = s;
+  slo[tid] = e;
+  __syncthreads();
+  {
+    // warp w sums right-hand side w over the CTA's threads
+    const int wq = tid >> 5;
+    if (wq < R) {
+      double t = 0.0;
+      for (int i = tid & 31; i < CS_THREADS; i += 32)
+        if ((cta * CS_THREADS + i) % Rp == wq) t += (double)shi[i] + (double)slo[i];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(FULL_MASK, t, o);
+      if ((tid & 31) == 0) sc->rr[cta][wq] = t;
+    }
+  }
+  cluster_sync();
+  // p = r + beta p, max |p|
+  double rn = 0.0;
+  if (live) {
+    for (int c = 0; c < CS_CTAS; ++c) rn += __ldcg(&sc->rr[c][q]);
+    const float be = (float)(ro > 0 ? rn / ro : 0.0);
+    float m = 0.f;
+    for (int j = gid; j < N; j += stride) {
+      const int it = j / Rp, a = it / KG, k0 = 8 * (it % KG);
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        if (k0 + k >= n) break;
+        const size_t o = ((size_t)a * n + k0 + k) * R + q;
+        float2 pv = p[o];
+        if (run) {
+          const float2 rv = r[o];
+          pv.x = rv.x + be * pv.x;
+          pv.y = rv.y + be * pv.y;
+          p[o] = pv;
+        }
+        m = fmaxf(m, fmaxf(fabsf(pv.x), fabsf(pv.y)));
+      }
+    }
+    if (m > 0.f) atomicMax(&sxm[q], __float_as_uint(m));
+  }
+  __syncthreads();
+  if (tid < R) sc->xm[cta][tid] = sxm[tid];
+  cluster_sync();
+  // the operand rows 4 q + {Re hi, Im hi, Re lo, Im lo} (zero for q >= R), as k_x_to_tc
+  unsigned xm = 0u;
+  if (live)
+    for (int c = 0; c < CS_CTAS; ++c) xm = max(xm, __ldcg(&sc->xm[c][q]));
+  const float scale = live ? pow2f(scale_exp(xm)) : 0.f;
+  if (gid < stride) {
+    for (int j = gid; j < N; j += stride) {
+      const int it = j / Rp, a = it / KG, kg = it % KG;
+      __align__(16) __half v[4][8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        float2 pv = make_float2(0.f, 0.f);
+        if (live && 8 * kg + k < n) pv = p[((size_t)a * n + 8 * kg + k) * R + q];
+        const float re = pv.x * scale, im = pv.y * scale;
+        const __half rh = __float2half_rn(re), ih = __float2half_rn(im);
+        v[0][k] = rh;
+        v[1][k] = ih;
+        v[2][k] = __float2half_rn(re - __half2float(rh));
+        v[3][k] = __float2half_rn(im - __half2float(ih));
+      }
+      char* tile = xtc + (size_t)a * (4 * Rp) * Kp * 2;
+#pragma unroll
+      for (int h = 0; h < 4; ++h) {
+        const int row = 4 * q + h;
+        *reinterpret_cast<uint4*>(tile + (size_t)(row / 8) * (Kp * 16) + kg * 128 + (row % 8) * 16) =
+            *reinterpret_cast<const uint4*>(v[h]);
+      }
+    }
+  }
+  // bookkeeping (nobody reads it in this launch any more)
+  if (gid < R) {
+    ctl->rr[par ^ 1][gid] = rn;
+    xmax[gid] = xm;
+  }
+  if (cta == 0) {
+    __syncthreads();
+    if (tid == 0) {
+      const int it = ctl->iter + 1;
+      ctl->iter = it;
+      int all = 1;
+      for (int i = 0; i < R; ++i) {
+        const double v = ctl->rr[par ^ 1][i];
+        if (!ctl->done[i] && (v <= ctl->stop[i] || it >= maxiter || !(v == v))) ctl->done[i] = 1;
+        all &= ctl->done[i];
+      }
+      ctl->all_done = all;
+    }
+  }
+}
+
+// Couplings split and one-launch step for grids whose pairs leave SMs idle and whose
+// vectors fit the cluster's items.
+static bool small_grid(const Coarse& A, const TcGeom& g, int& nsplit) {
+  const int npairs = (int)((A.Vc + g.sites - 1) / g.sites), slots = 2 * device_sms();
+  nsplit = std::max(1, std::min(8, slots / npairs));
+  const int threads = CS_CTAS * CS_THREADS / g.Rp * g.Rp;
+  return A.Vc * (g.Kp / 8) * g.Rp <= (size_t)threads * CS_ITEMS;
+}
+
 int coarse_cg_tc(Ctx& c, Coarse& A, int R, const void* rhs, void* sol, double tol, int maxiter, double shift) {
   coarse_tc_prepare(c, A);
   const size_t ne = A.Vc * A.nvec;
   const size_t nc = ne * R;
-  A.work.ensure(3 * nc * sizeof(float2));
-  A.ctl.ensure(sizeof(CCtlT));
+  const TcGeom g = tc_geom(A.nvec, R, tc_parts(A));
+  int nsplit = 1;
+  const bool small = small_grid(A, g, nsplit);
+  if (!small) nsplit = 1;
+  A.work.ensure((2 + nsplit) * nc * sizeof(float2));
+  A.ctl.ensure(sizeof(CCtlT) + sizeof(CgStepScratch));
   float2* r = A.work.as<float2>();
   float2* p = r + nc;
   float2* w = p + nc;
   CCtlT* ctl = A.ctl.as<CCtlT>();
+  CgStepScratch* sc = reinterpret_cast<CgStepScratch*>(ctl + 1);
   unsigned* xmax = A.tcs.as<TcState>()->xmax;
   const int* skip = &ctl->all_done;
   const unsigned ge = (unsigned)((ne + 255) / 256);
@@ -813,7 +1002,15 @@ int coarse_cg_tc(Ctx& c, Coarse& A, int R, const void* rhs, void* sol, double to
                                        make_reduction(c, ge, RMAX, &ctl->rr[0][0], 0));
   k_cgt_start<<<1, 1, 0, c.stream>>>(ctl, R, tol, maxiter);
   c.launches += 2;
+  if (small) coarse_tc_to_b(c, A, R, p, xmax, skip);   // afterwards the step kernel writes the operand
   auto iteration = [&](int par) {
+    if (small) {
+      launch_tc(c, A, R, p, w, xmax, skip, &ctl->pAp[0], shift, c.tc_force ? c.tc_force : 2, nullptr, nsplit);
+      k_cgt_step<<<CS_CTAS, CS_THREADS, 0, c.stream>>>((float2*)sol, r, p, w, nsplit, nc, (int)A.Vc, A.nvec, R, g.Rp, g.Kp,
+                                                       A.xtc.as<char>(), ctl, sc, par, maxiter, xmax);
+      ++c.launches;
+      return;
+    }
     coarse_tc_to_b(c, A, R, p, xmax, skip);
     coarse_tc_apply(c, A, R, p, w, xmax, skip, &ctl->pAp[0], shift);
     k_cgt_update<<<ge, 256, 0, c.stream>>>((float2*)sol, r, p, w, ne, R, ctl, par, xmax,
