@@ -152,11 +152,16 @@ __global__ void k_site_scale(const AT* __restrict__ A, int n, int* sexp) {
 
 // A ([a][l][k][j] complex, FP16 or FP32) -> tiled operand, one 16-byte row segment per
 // thread: element (m, k) (m < rows, k < 8 kgs) of part p of block (a, l) at byte
-// (blk parts + p) a_gbytes + (m/8) sbo + (k/8) lbo + (m%8) 16 + (k%8) 2; part 0 = hi,
-// part 1 = lo.
+// tc_block(a, l, p) a_gbytes + (m/8) sbo + (k/8) lbo + (m%8) 16 + (k%8) 2; part 0 = hi,
+// part 1 = lo.  The sites of an MMA lie side by side, part by part, coupling by
+// coupling: a stage's A is one contiguous run.
+__device__ __forceinline__ size_t tc_block(size_t a, int l, int p, int sites, int parts) {
+  return ((a / sites * 81 + l) * parts + p) * sites + a % sites;
+}
 template <typename AT>
 __global__ void k_a_to_tc(const AT* __restrict__ A, uint4* __restrict__ Atc, size_t nblk, int n, int rows, int kgs,
-                          uint32_t a_gbytes, uint32_t lbo, uint32_t sbo, int parts, const int* __restrict__ sexp) {
+                          uint32_t a_gbytes, uint32_t lbo, uint32_t sbo, int sites, int parts,
+                          const int* __restrict__ sexp) {
   const int KG = kgs;
   const size_t per = (size_t)rows * KG;
   const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -179,10 +184,12 @@ __global__ void k_a_to_tc(const AT* __restrict__ A, uint4* __restrict__ Atc, siz
     hi[q] = __float2half_rn(x);
     lo[q] = __float2half_rn(x - __half2float(hi[q]));
   }
-  char* dst = reinterpret_cast<char*>(Atc) + blk * parts * (size_t)a_gbytes + (size_t)(m / 8) * sbo +
-              (size_t)kg * lbo + (m % 8) * 16;
-  *reinterpret_cast<uint4*>(dst) = *reinterpret_cast<const uint4*>(hi);
-  if (parts == 2) *reinterpret_cast<uint4*>(dst + a_gbytes) = *reinterpret_cast<const uint4*>(lo);
+  const size_t a = blk / 81;
+  const int l = (int)(blk % 81);
+  char* dst = reinterpret_cast<char*>(Atc) + (size_t)(m / 8) * sbo + (size_t)kg * lbo + (m % 8) * 16;
+  *reinterpret_cast<uint4*>(dst + tc_block(a, l, 0, sites, parts) * a_gbytes) = *reinterpret_cast<const uint4*>(hi);
+  if (parts == 2)
+    *reinterpret_cast<uint4*>(dst + tc_block(a, l, 1, sites, parts) * a_gbytes) = *reinterpret_cast<const uint4*>(lo);
 }
 
 // X (FP32 complex [a][k][r]) -> tiled B operand of every coarse site: thread
@@ -356,46 +363,48 @@ __global__ void __launch_bounds__(TC_THREADS, 2) k_capply_tc(TcArgs g, Reduction
   if (w == 0) {
     // ---- producer: bulk copies of A blocks and neighbour B tiles --------------------
     // The whole warp first fetches the pair's 81 (or 162) neighbour indices into
-    // shared memory in one round trip; lane 0 then issues the copies without a
-    // dependent global load in front of every stage.
+    // shared memory in one round trip.  Then every lane of the first few issues one
+    // copy of a stage, its source advancing by itself: lane 0 the A run of both sites
+    // (one site with K padding: one lane per part), the next lanes the B tiles.  With
+    // one lane issuing all four to six copies and dividing for its ring position, a
+    // stage took 0.65 to 0.82 us whatever its size (24^3 x 48, FP16: 244 us an apply).
     __shared__ int snb[2 * 81];
-    uint32_t it = 0;
+    const int nA = g.sites == 2 ? 1 : g.parts, ncopy = nA + g.sites;
+    const uint32_t abytes = g.sites == 2 ? 2u * g.parts * g.a_gbytes : g.a_gbytes;
+    const size_t astep = (size_t)g.sites * g.parts * g.a_gbytes;     // one coupling of a pair
+    const uint32_t doff = lane < nA ? (uint32_t)lane * g.a_sbytes
+                                    : (uint32_t)(g.sites * g.parts) * g.a_sbytes + (uint32_t)(lane - nA) * g.b_bytes;
+    const uint32_t bytes = lane < nA ? abytes : g.b_bytes;
+    uint32_t it = 0, s = 0, ph = 0;
     bool ok = true;
     for (int p = blockIdx.x; ok && p < items; p += gridDim.x) {
-      const int s0 = p / g.nsplit * g.sites;
+      const int pair = p / g.nsplit, s0 = pair * g.sites;
       const int l0 = split_begin(p % g.nsplit, g.nsplit), l1 = split_begin(p % g.nsplit + 1, g.nsplit);
       const int s1 = min(s0 + 1, g.Vc - 1);
       for (int q = lane; q < g.sites * 81; q += 32)
         snb[q] = __ldg(g.cnbr + (size_t)(q < 81 ? s0 : s1) * 81 + q % 81);
       __syncwarp();
-      if (lane == 0) {
-        for (int l = l0; l < l1; ++l, ++it) {
-          const int s = (int)(it % (uint32_t)g.stages);
-          const uint32_t ph = (it / (uint32_t)g.stages) & 1u;
-          if (!tc::mbar_wait(TC_EMPTY(s), ph ^ 1u)) {
-            ok = false;
-            atomicOr(g.err, 1u);
-            break;
-          }
-          tc::mbar_arrive_expect_tx(TC_FULL(s), g.copy_bytes);
-          const uint32_t dst = ring + (uint32_t)s * stage_bytes;
-          // stage: [part 0: site 0, site 1][part 1: site 0, site 1][B site 0][B site 1]
-          for (int pp = 0; pp < g.parts; ++pp)
-            for (int si = 0; si < g.sites; ++si) {
-              const size_t blk = (size_t)(si ? s1 : s0) * 81 + l;
-              tc::bulk_g2s(dst + (pp * g.sites + si) * g.a_sbytes,
-                           reinterpret_cast<const char*>(g.Atc) + (blk * g.parts + pp) * g.a_gbytes, g.a_gbytes,
-                           TC_FULL(s));
-            }
-          for (int si = 0; si < g.sites; ++si) {
-            const int nb = snb[si * 81 + l];
-            tc::bulk_g2s(dst + g.sites * g.parts * g.a_sbytes + si * g.b_bytes,
-                         reinterpret_cast<const char*>(g.xtc) + (size_t)nb * g.b_bytes, g.b_bytes, TC_FULL(s));
-          }
+      const char* src = reinterpret_cast<const char*>(g.Atc) + ((size_t)pair * 81 + l0) * astep + (size_t)lane * g.a_gbytes;
+      const int* nb = snb + (lane >= nA && lane < ncopy ? (lane - nA) * 81 : 0);
+      for (int l = l0; l < l1; ++l, ++it) {
+        ok = __all_sync(FULL_MASK, tc::mbar_wait(TC_EMPTY(s), ph ^ 1u));
+        if (!ok) {
+          if (lane == 0) atomicOr(g.err, 1u);
+          break;
+        }
+        if (lane == 0) tc::mbar_arrive_expect_tx(TC_FULL(s), g.copy_bytes);
+        // stage: [part 0: site 0, site 1][part 1: site 0, site 1][B site 0][B site 1]
+        if (lane < ncopy)
+          tc::bulk_g2s(ring + s * stage_bytes + doff,
+                       lane < nA ? src : reinterpret_cast<const char*>(g.xtc) + (size_t)nb[l] * g.b_bytes, bytes,
+                       TC_FULL(s));
+        src += astep;
+        if (++s == (uint32_t)g.stages) {
+          s = 0;
+          ph ^= 1u;
         }
       }
-      ok = __shfl_sync(FULL_MASK, ok ? 1 : 0, 0) != 0;
-      __syncwarp();   // lane 0 is done with snb before the next pair overwrites it
+      __syncwarp();   // every lane is done with snb before the next pair overwrites it
     }
     if (lane == 0) {
       // every copy issued has to land before the CTA exits
@@ -406,7 +415,7 @@ __global__ void __launch_bounds__(TC_THREADS, 2) k_capply_tc(TcArgs g, Reduction
   } else if (w == 1) {
     // ---- MMA issuer ------------------------------------------------------------------
     if (lane == 0) {
-      uint32_t it = 0;
+      uint32_t s = 0, ph = 0;
       int np = 0;
       bool ok = true;
       const uint32_t sbo = (uint32_t)g.Kp * 16u;
@@ -418,16 +427,14 @@ __global__ void __launch_bounds__(TC_THREADS, 2) k_capply_tc(TcArgs g, Reduction
           break;
         }
         tc::fence_after_sync();
-        for (int l = l0; l < l1; ++l, ++it) {
-          const int s = (int)(it % (uint32_t)g.stages);
-          const uint32_t ph = (it / (uint32_t)g.stages) & 1u;
+        for (int l = l0; l < l1; ++l) {
           if (!tc::mbar_wait(TC_FULL(s), ph)) {
             ok = false;
             atomicOr(g.err, 8u);
             break;
           }
           tc::fence_after_sync();
-          const uint32_t abase = ring + (uint32_t)s * stage_bytes;
+          const uint32_t abase = ring + s * stage_bytes;
           const uint32_t bbase = abase + g.sites * g.parts * g.a_sbytes;
           for (int ks = 0; ks < g.Kp / 16; ++ks) {
             const uint64_t bd = tc::smem_desc(bbase + 256u * ks, 128u, sbo);
@@ -438,6 +445,10 @@ __global__ void __launch_bounds__(TC_THREADS, 2) k_capply_tc(TcArgs g, Reduction
             }
           }
           tc::mma_commit(TC_EMPTY(s));
+          if (++s == (uint32_t)g.stages) {
+            s = 0;
+            ph ^= 1u;
+          }
         }
         if (ok) tc::mma_commit(ACC_FULL);
       }
@@ -523,7 +534,9 @@ void coarse_tc_prepare(Ctx& c, Coarse& A) {
   const int parts = tc_parts(A);
   const TcGeom g = tc_geom(A.nvec, 1, parts);
   const size_t nblk = A.Vc * 81;
-  A.Atc.ensure(nblk * parts * g.a_gbytes);
+  const size_t abytes = (A.Vc + g.sites - 1) / g.sites * g.sites * 81 * parts * (size_t)g.a_gbytes;
+  A.Atc.ensure(abytes);
+  if (A.Vc % g.sites) HDCG_CUDA(cudaMemsetAsync(A.Atc.p, 0, abytes, c.stream));   // the last pair's missing site
   A.sexp.ensure(A.Vc * sizeof(int));
   A.tcs.ensure(sizeof(TcState));
   HDCG_CUDA(cudaMemsetAsync(A.tcs.p, 0, sizeof(TcState), c.stream));
@@ -531,12 +544,12 @@ void coarse_tc_prepare(Ctx& c, Coarse& A) {
   if (A.prec == HDCG_F32) {
     k_site_scale<float2><<<(unsigned)A.Vc, 256, 0, c.stream>>>(A.A.as<float2>(), A.nvec, A.sexp.as<int>());
     k_a_to_tc<float2><<<(unsigned)((nt + 255) / 256), 256, 0, c.stream>>>(
-        A.A.as<float2>(), A.Atc.as<uint4>(), nblk, A.nvec, g.rows, g.kgs, g.a_gbytes, g.lbo_a, g.sbo_a, parts,
+        A.A.as<float2>(), A.Atc.as<uint4>(), nblk, A.nvec, g.rows, g.kgs, g.a_gbytes, g.lbo_a, g.sbo_a, g.sites, parts,
         A.sexp.as<int>());
   } else {
     k_site_scale<__half2><<<(unsigned)A.Vc, 256, 0, c.stream>>>(A.A.as<__half2>(), A.nvec, A.sexp.as<int>());
     k_a_to_tc<__half2><<<(unsigned)((nt + 255) / 256), 256, 0, c.stream>>>(
-        A.A.as<__half2>(), A.Atc.as<uint4>(), nblk, A.nvec, g.rows, g.kgs, g.a_gbytes, g.lbo_a, g.sbo_a, parts,
+        A.A.as<__half2>(), A.Atc.as<uint4>(), nblk, A.nvec, g.rows, g.kgs, g.a_gbytes, g.lbo_a, g.sbo_a, g.sites, parts,
         A.sexp.as<int>());
   }
   HDCG_CUDA(cudaGetLastError());
@@ -846,33 +859,44 @@ __global__ void __cluster_dims__(CS_CTAS, 1, 1) __launch_bounds__(CS_THREADS)
     const double pap = ctl->pAp[q];
     const float al = (float)(pap > 0 ? ro / pap : 0.0);
     for (int j = gid; j < N; j += stride) {
-      const int it = j / Rp, a = it / KG, k0 = 8 * (it % KG);
+      const int it = j / Rp, a = it / KG, k0 = 8 * (it % KG), kc = min(8, n - k0);
+      const size_t o0 = ((size_t)a * n + k0) * R + q;
+      // every load of the item in flight before the first use
+      float2 rv[8], pv[8], wv[8], xv[8];
 #pragma unroll
       for (int k = 0; k < 8; ++k) {
-        if (k0 + k >= n) break;
-        const size_t o = ((size_t)a * n + k0 + k) * R + q;
-        float2 rv = r[o];
-        if (run) {
-          const float2 pv = p[o];
-          float2 wv = w[o], xv = x[o];
-          for (int t = 1; t < nsplit; ++t) {
-            const float2 u = w[t * part + o];
-            wv.x += u.x;
-            wv.y += u.y;
-          }
-          xv.x += al * pv.x;
-          xv.y += al * pv.y;
-          rv.x -= al * wv.x;
-          rv.y -= al * wv.y;
-          x[o] = xv;
-          r[o] = rv;
+        const size_t o = o0 + (size_t)min(k, kc - 1) * R;
+        rv[k] = r[o];
+        pv[k] = p[o];
+        wv[k] = w[o];
+        xv[k] = x[o];
+      }
+      for (int t = 1; t < nsplit; ++t)
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          const float2 u = w[t * part + o0 + (size_t)min(k, kc - 1) * R];
+          wv[k].x += u.x;
+          wv[k].y += u.y;
         }
 #pragma unroll
-        for (int c = 0; c < 2; ++c) {
-          const float v = c ? rv.y : rv.x, sq = __fmul_rn(v, v), d = __fmaf_rn(v, v, -sq);
-          float u;
-          two_sum(s, sq, s, u);
-          e = __fadd_rn(e, __fadd_rn(u, d));
+      for (int k = 0; k < 8; ++k) {
+        if (k < kc) {
+          if (run) {
+            const size_t o = o0 + (size_t)k * R;
+            xv[k].x += al * pv[k].x;
+            xv[k].y += al * pv[k].y;
+            rv[k].x -= al * wv[k].x;
+            rv[k].y -= al * wv[k].y;
+            x[o] = xv[k];
+            r[o] = rv[k];
+          }
+#pragma unroll
+          for (int c = 0; c < 2; ++c) {
+            const float v = c ? rv[k].y : rv[k].x, sq = __fmul_rn(v, v), d = __fmaf_rn(v, v, -sq);
+            float u;
+            two_sum(s, sq, s, u);
+            e = __fadd_rn(e, __fadd_rn(u, d));
+          }
         }
       }
     }
@@ -900,19 +924,25 @@ __global__ void __cluster_dims__(CS_CTAS, 1, 1) __launch_bounds__(CS_THREADS)
     const float be = (float)(ro > 0 ? rn / ro : 0.0);
     float m = 0.f;
     for (int j = gid; j < N; j += stride) {
-      const int it = j / Rp, a = it / KG, k0 = 8 * (it % KG);
+      const int it = j / Rp, a = it / KG, k0 = 8 * (it % KG), kc = min(8, n - k0);
+      const size_t o0 = ((size_t)a * n + k0) * R + q;
+      float2 rv[8], pv[8];
 #pragma unroll
       for (int k = 0; k < 8; ++k) {
-        if (k0 + k >= n) break;
-        const size_t o = ((size_t)a * n + k0 + k) * R + q;
-        float2 pv = p[o];
-        if (run) {
-          const float2 rv = r[o];
-          pv.x = rv.x + be * pv.x;
-          pv.y = rv.y + be * pv.y;
-          p[o] = pv;
+        const size_t o = o0 + (size_t)min(k, kc - 1) * R;
+        rv[k] = r[o];
+        pv[k] = p[o];
+      }
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        if (k < kc) {
+          if (run) {
+            pv[k].x = rv[k].x + be * pv[k].x;
+            pv[k].y = rv[k].y + be * pv[k].y;
+            p[o0 + (size_t)k * R] = pv[k];
+          }
+          m = fmaxf(m, fmaxf(fabsf(pv[k].x), fabsf(pv[k].y)));
         }
-        m = fmaxf(m, fmaxf(fabsf(pv.x), fabsf(pv.y)));
       }
     }
     if (m > 0.f) atomicMax(&sxm[q], __float_as_uint(m));
