@@ -5,6 +5,8 @@
 // hence different chunking) line up.  Every reduction accumulates in FP64
 // (per-thread FP32/FP64 partial over 24 reals, then FP64 warp / block / grid
 // sums in a fixed order: two runs give bit-identical results).
+#include <type_traits>
+
 #include "blas.cuh"
 
 namespace hdcg {
@@ -254,21 +256,34 @@ void zero_field(Ctx& c, uint4* f, int prec, size_t nf) {
 // ---------------------------------------------------------------------------
 // reductions
 // ---------------------------------------------------------------------------
+// the NV partial sums of a thread into the grid reduction: FP32 partials through
+// double-float warp sums, FP64 ones in FP64
+template <int NV, typename R>
+__device__ __forceinline__ void reduce_partials(R (&s)[NV], const Reduction& red) {
+  if constexpr (std::is_same<R, float>::value) {
+    float lo[NV];
+#pragma unroll
+    for (int i = 0; i < NV; ++i) lo[i] = 0.f;
+    grid_reduce_pairs<NV>(s, lo, red);
+  } else {
+    grid_reduce<NV>(s, red);
+  }
+}
 template <typename S>
 __global__ void k_norm2(const uint4* __restrict__ a, size_t n5, Reduction red, size_t fstride) {
   using R = typename Store<S>::real;
   a += blockIdx.y * fstride;
   const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  double v[1] = {0.0};
+  R v[1] = {0};
   if (t < n5) {
     R x[24];
     load_spinor<S, R>(a, t, n5, x);
     R s = 0;
 #pragma unroll
     for (int i = 0; i < 24; ++i) s += x[i] * x[i];
-    v[0] = (double)s;
+    v[0] = s;
   }
-  grid_reduce<1>(v, red);
+  reduce_partials<1>(v, red);
 }
 
 template <typename S>
@@ -338,7 +353,10 @@ __global__ void k_update_xr(uint4* x, const uint4* __restrict__ p, uint4* r, con
                             size_t n5, ScalarRef al, int sign_x, Reduction red) {
   using Rx = typename Store<Sx>::real;
   using R = typename Store<S>::real;
-  const double alpha = ratio(al.num, al.den0, al.den1, al.lam);
+  __shared__ double s_alpha;   // FP64 divisions and roots: one per CTA, not one per thread
+  if (threadIdx.x == 0) s_alpha = ratio(al.num, al.den0, al.den1, al.lam);
+  __syncthreads();
+  const double alpha = s_alpha;
   const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   double v[1] = {0.0};
   if (t < n5) {
@@ -372,15 +390,17 @@ __global__ void k_update_p(uint4* p, const uint4* __restrict__ y, size_t n5, Sca
   const int rr = blockIdx.y;
   p += rr * fstride;
   y += rr * fstride;
-  double beta = 0.0;
-  {
+  __shared__ double s_beta;
+  if (threadIdx.x == 0) {
     double n = be.num[rr * be.stride];
     if (be.den1) n -= be.den1[rr * be.stride];  // n1 stored in den1 slot for beta
     const double d = be.den0[rr];
-    beta = d != 0.0 ? n / d : 0.0;
+    s_beta = d != 0.0 ? n / d : 0.0;
   }
+  __syncthreads();
+  const double beta = s_beta;
   const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  double v[1] = {0.0};
+  R v[1] = {0};
   if (t < n5) {
     R pv[24], yv[24];
     load_spinor<S, R>(p, t, n5, pv);
@@ -393,9 +413,9 @@ __global__ void k_update_p(uint4* p, const uint4* __restrict__ y, size_t n5, Sca
       s += pv[i] * pv[i];
     }
     store_spinor<S, R>(p, t, n5, pv);
-    v[0] = (double)s;
+    v[0] = s;
   }
-  if (do_red) grid_reduce<1>(v, red);
+  if (do_red) reduce_partials<1>(v, red);
 }
 
 // res[0] = Re<a, b>, res[1] = Re<a, c> (c may be null)
@@ -408,7 +428,7 @@ __global__ void k_redot2(const uint4* __restrict__ a, const uint4* __restrict__ 
   b += ro;
   if (cc) cc += ro;
   const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  double v[2] = {0.0, 0.0};
+  R v[2] = {0, 0};
   if (t < n5) {
     R av[24], bv[24];
     load_spinor<S, R>(a, t, n5, av);
@@ -422,10 +442,10 @@ __global__ void k_redot2(const uint4* __restrict__ a, const uint4* __restrict__ 
 #pragma unroll
       for (int i = 0; i < 24; ++i) s1 += av[i] * cv[i];
     }
-    v[0] = (double)s0;
-    v[1] = (double)s1;
+    v[0] = s0;
+    v[1] = s1;
   }
-  grid_reduce<2>(v, red);
+  reduce_partials<2>(v, red);
 }
 
 // hi += lo ; lo = 0
@@ -472,10 +492,16 @@ __global__ void k_scale_dev(const uint4* __restrict__ x, uint4* y, size_t n5, co
                             const double* den, int inv) {
   using R = typename Store<S>::real;
   const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  __shared__ double s_scale;
+  if (threadIdx.x == 0) {
+    double q = *den > 0 ? *num / *den : 0.0;
+    double s = sqrt(q);
+    if (inv) s = s > 0 ? 1.0 / s : 0.0;
+    s_scale = s;
+  }
+  __syncthreads();
   if (t >= n5) return;
-  double q = *den > 0 ? *num / *den : 0.0;
-  double s = sqrt(q);
-  if (inv) s = s > 0 ? 1.0 / s : 0.0;
+  const double s = s_scale;
   R v[24];
   load_spinor<S, R>(x, t, n5, v);
 #pragma unroll
@@ -493,11 +519,16 @@ __global__ void k_convert_scaled(const uint4* __restrict__ in, uint4* __restrict
   in += rr * fsi;
   out += rr * fso;
   const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  __shared__ double s_scale;
+  if (threadIdx.x == 0) {
+    const double nv = num[0], dv = den[rr];
+    const double q = (dv > 0.0 && nv > 0.0) ? nv / dv : 1.0;
+    const double sc = sqrt(q);
+    s_scale = inv ? 1.0 / sc : sc;
+  }
+  __syncthreads();
   if (t >= n5) return;
-  const double nv = num[0], dv = den[rr];
-  const double q = (dv > 0.0 && nv > 0.0) ? nv / dv : 1.0;
-  double sc = sqrt(q);
-  if (inv) sc = 1.0 / sc;
+  const double sc = s_scale;
   Ri v[24];
   load_spinor<Si, Ri>(in, t, n5, v);
   Ro w[24];

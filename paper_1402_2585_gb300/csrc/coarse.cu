@@ -469,13 +469,6 @@ __device__ __forceinline__ void load_complex(const uint4* __restrict__ f, int z,
   }
 }
 
-// a float as a double without the FP64 pipe's conversion
-__device__ __forceinline__ double widen(float x) {
-  double d;
-  return widen_float(x, d) ? d : (double)x;
-}
-__device__ __forceinline__ double widen(double x) { return x; }
-
 // Sums the 32 values of every lane over the warp: lane l returns the total of
 // v[l].  31 additions instead of 160 for a butterfly per value (the FP64 pipe
 // does two lanes per clock and SM).
@@ -1292,8 +1285,10 @@ template <typename R>
 __global__ void k_ccg_update(typename CV<R>::T* x, typename CV<R>::T* r, const typename CV<R>::T* p,
                              const typename CV<R>::T* w, size_t nc, const CCtl* ctl, int par, Reduction red) {
   if (ctl->done) return;
-  const double alpha = ctl->pAp > 0 ? ctl->rr[par] / ctl->pAp : 0.0;
-  const R al = (R)alpha;
+  __shared__ double s_alpha;
+  if (threadIdx.x == 0) s_alpha = ctl->pAp > 0 ? ctl->rr[par] / ctl->pAp : 0.0;
+  __syncthreads();
+  const R al = (R)s_alpha;
   const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   double v[1] = {0.0};
   if (t < nc) {
@@ -1319,15 +1314,24 @@ __global__ void k_ccg_update(typename CV<R>::T* x, typename CV<R>::T* r, const t
 template <typename R>
 __global__ void k_ccg_p(typename CV<R>::T* p, const typename CV<R>::T* r, size_t nc, CCtl* ctl, int par,
                         int maxiter) {
-  if (ctl->done) return;
-  const double rr_old = ctl->rr[par], rr_new = ctl->rr[par ^ 1];
+  // one decision per CTA (CTA 0 sets done below while others may still start)
+  __shared__ double s_beta;
+  __shared__ int s_done;
+  const double rr_new = ctl->rr[par ^ 1];
+  if (threadIdx.x == 0) {
+    const double rr_old = ctl->rr[par];
+    s_done = ctl->done;
+    s_beta = rr_old > 0 ? rr_new / rr_old : 0.0;
+  }
+  __syncthreads();
+  if (s_done) return;
   const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t == 0) {
     const int it = ctl->iter + 1;
     ctl->iter = it;
     if (rr_new <= ctl->stop || it >= maxiter || !(rr_new == rr_new)) ctl->done = 1;
   }
-  const R beta = (R)(rr_old > 0 ? rr_new / rr_old : 0.0);
+  const R beta = (R)s_beta;
   if (t < nc) {
     typename CV<R>::T pv = p[t];
     const typename CV<R>::T rv = r[t];
@@ -1910,6 +1914,12 @@ __global__ void k_ccgm_update(typename CV<R_>::T* x, typename CV<R_>::T* r, cons
                               const typename CV<R_>::T* w, size_t ne, int R, size_t nc, const CCtlM* ctl, int par,
                               Reduction red) {
   if (ctl->all_done) return;
+  __shared__ R_ s_al[RMAX];
+  if (threadIdx.x < R) {
+    const double pap = ctl->pAp[threadIdx.x];
+    s_al[threadIdx.x] = (R_)((!ctl->done[threadIdx.x] && pap > 0) ? ctl->rr[par][threadIdx.x] / pap : 0.0);
+  }
+  __syncthreads();
   const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   double v[RMAX];
 #pragma unroll
@@ -1918,8 +1928,7 @@ __global__ void k_ccgm_update(typename CV<R_>::T* x, typename CV<R_>::T* r, cons
 #pragma unroll
     for (int q = 0; q < RMAX; ++q) {
       if (q < R) {
-        const double pap = ctl->pAp[q];
-        const R_ al = (R_)((!ctl->done[q] && pap > 0) ? ctl->rr[par][q] / pap : 0.0);
+        const R_ al = s_al[q];
         const size_t e = t * R + q;
         typename CV<R_>::T xv = x[e], rv = r[e];
         const typename CV<R_>::T pv = p[e];
@@ -1946,13 +1955,18 @@ template <typename R_>
 __global__ void k_ccgm_p(typename CV<R_>::T* p, const typename CV<R_>::T* r, size_t ne, int R, CCtlM* ctl, int par,
                          int maxiter) {
   if (ctl->all_done) return;
+  __shared__ R_ s_be[RMAX];
+  if (threadIdx.x < R) {
+    const double ro = ctl->rr[par][threadIdx.x], rn = ctl->rr[par ^ 1][threadIdx.x];
+    s_be[threadIdx.x] = (R_)(ro > 0 ? rn / ro : 0.0);
+  }
+  __syncthreads();
   const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t < ne) {
 #pragma unroll
     for (int q = 0; q < RMAX; ++q) {
       if (q < R && !ctl->done[q]) {
-        const double ro = ctl->rr[par][q], rn = ctl->rr[par ^ 1][q];
-        const R_ beta = (R_)(ro > 0 ? rn / ro : 0.0);
+        const R_ beta = s_be[q];
         const size_t e = t * R + q;
         typename CV<R_>::T pv = p[e];
         const typename CV<R_>::T rv = r[e];

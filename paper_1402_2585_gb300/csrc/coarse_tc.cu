@@ -386,25 +386,26 @@ __global__ void __launch_bounds__(TC_THREADS, 2) k_capply_tc(TcArgs g, Reduction
       __syncwarp();
       const char* src = reinterpret_cast<const char*>(g.Atc) + ((size_t)pair * 81 + l0) * astep + (size_t)lane * g.a_gbytes;
       const int* nb = snb + (lane >= nA && lane < ncopy ? (lane - nA) * 81 : 0);
-      for (int l = l0; l < l1; ++l, ++it) {
-        ok = __all_sync(FULL_MASK, tc::mbar_wait(TC_EMPTY(s), ph ^ 1u));
-        if (!ok) {
-          if (lane == 0) atomicOr(g.err, 1u);
-          break;
-        }
-        if (lane == 0) tc::mbar_arrive_expect_tx(TC_FULL(s), g.copy_bytes);
-        // stage: [part 0: site 0, site 1][part 1: site 0, site 1][B site 0][B site 1]
-        if (lane < ncopy)
+      if (lane < ncopy) {
+        for (int l = l0; l < l1; ++l, ++it) {
+          if (!tc::mbar_wait(TC_EMPTY(s), ph ^ 1u)) {
+            ok = false;
+            atomicOr(g.err, 1u);
+            break;
+          }
+          if (lane == 0) tc::mbar_arrive_expect_tx(TC_FULL(s), g.copy_bytes);
+          // stage: [part 0: site 0, site 1][part 1: site 0, site 1][B site 0][B site 1]
           tc::bulk_g2s(ring + s * stage_bytes + doff,
                        lane < nA ? src : reinterpret_cast<const char*>(g.xtc) + (size_t)nb[l] * g.b_bytes, bytes,
                        TC_FULL(s));
-        src += astep;
-        if (++s == (uint32_t)g.stages) {
-          s = 0;
-          ph ^= 1u;
+          src += astep;
+          if (++s == (uint32_t)g.stages) {
+            s = 0;
+            ph ^= 1u;
+          }
         }
       }
-      __syncwarp();   // every lane is done with snb before the next pair overwrites it
+      ok = __all_sync(FULL_MASK, ok);   // every lane is done with snb before the next pair overwrites it
     }
     if (lane == 0) {
       // every copy issued has to land before the CTA exits
@@ -418,7 +419,9 @@ __global__ void __launch_bounds__(TC_THREADS, 2) k_capply_tc(TcArgs g, Reduction
       uint32_t s = 0, ph = 0;
       int np = 0;
       bool ok = true;
-      const uint32_t sbo = (uint32_t)g.Kp * 16u;
+      const uint64_t bdesc = tc::smem_desc(0, 128u, (uint32_t)g.Kp * 16u), adesc = tc::smem_desc(0, g.lbo_a, g.sbo_a);
+      const int ksteps = g.Kp / 16;
+      const uint32_t pstep = g.sites * g.a_sbytes;
       for (int p = blockIdx.x; ok && p < items; p += gridDim.x, ++np) {
         const int l0 = split_begin(p % g.nsplit, g.nsplit), l1 = split_begin(p % g.nsplit + 1, g.nsplit);
         if (np > 0 && !tc::mbar_wait(ACC_EMPTY, (uint32_t)(np - 1) & 1u)) {
@@ -436,11 +439,12 @@ __global__ void __launch_bounds__(TC_THREADS, 2) k_capply_tc(TcArgs g, Reduction
           tc::fence_after_sync();
           const uint32_t abase = ring + s * stage_bytes;
           const uint32_t bbase = abase + g.sites * g.parts * g.a_sbytes;
-          for (int ks = 0; ks < g.Kp / 16; ++ks) {
-            const uint64_t bd = tc::smem_desc(bbase + 256u * ks, 128u, sbo);
+          // addresses below 256 KB: a step is an addition to the descriptor's low word
+          const uint64_t bd0 = bdesc | (bbase >> 4), ad0 = adesc | (abase >> 4);
+          for (int ks = 0; ks < ksteps; ++ks) {
+            const uint64_t bd = bd0 + 16u * ks;
             for (int p = 0; p < g.parts; ++p) {
-              const uint64_t ad =
-                  tc::smem_desc(abase + p * g.sites * g.a_sbytes + 2u * g.lbo_a * ks, g.lbo_a, g.sbo_a);
+              const uint64_t ad = ad0 + ((p * pstep + 2u * g.lbo_a * ks) >> 4);
               tc::mma_f16(tmem, ad, bd, g.idesc, (l != l0 || (ks | p) != 0) ? 1u : 0u);
             }
           }
@@ -741,9 +745,15 @@ __global__ void k_cgt_update(float2* x, float2* r, const float2* __restrict__ p,
   const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t == 0)
     for (int q = 0; q < RMAX; ++q) xmax[q] = 0u;
-  double v[RMAX];
+  __shared__ float s_al[RMAX];   // one FP64 division per right-hand side and CTA
+  if (threadIdx.x < R) {
+    const double pap = ctl->pAp[threadIdx.x];
+    s_al[threadIdx.x] = (float)(pap > 0 ? ctl->rr[par][threadIdx.x] / pap : 0.0);
+  }
+  __syncthreads();
+  float hi[RMAX], lo[RMAX];
 #pragma unroll
-  for (int q = 0; q < RMAX; ++q) v[q] = 0.0;
+  for (int q = 0; q < RMAX; ++q) hi[q] = lo[q] = 0.f;
   if (t < ne) {
 #pragma unroll
     for (int q = 0; q < RMAX; ++q) {
@@ -751,8 +761,7 @@ __global__ void k_cgt_update(float2* x, float2* r, const float2* __restrict__ p,
         const size_t e = t * R + q;
         float2 rv = r[e];
         if (!ctl->done[q]) {
-          const double pap = ctl->pAp[q];
-          const float al = (float)(pap > 0 ? ctl->rr[par][q] / pap : 0.0);
+          const float al = s_al[q];
           const float2 pv = p[e], wv = w[e];
           float2 xv = x[e];
           xv.x += al * pv.x;
@@ -762,11 +771,12 @@ __global__ void k_cgt_update(float2* x, float2* r, const float2* __restrict__ p,
           x[e] = xv;
           r[e] = rv;
         }
-        v[q] = (double)rv.x * rv.x + (double)rv.y * rv.y;
+        add_square(hi[q], lo[q], rv.x);
+        add_square(hi[q], lo[q], rv.y);
       }
     }
   }
-  grid_reduce<RMAX>(v, red, R);
+  grid_reduce_pairs<RMAX>(hi, lo, red, R);
 }
 
 // p = r + beta p for the right-hand sides still running; max|p| of every right-hand side
@@ -774,6 +784,12 @@ __global__ void k_cgt_p(float2* p, const float2* __restrict__ r, size_t ne, int 
                         unsigned* xmax) {
   if (ctl->all_done) return;
   const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  __shared__ float s_be[RMAX];
+  if (threadIdx.x < R) {
+    const double ro = ctl->rr[par][threadIdx.x], rn = ctl->rr[par ^ 1][threadIdx.x];
+    s_be[threadIdx.x] = (float)(ro > 0 ? rn / ro : 0.0);
+  }
+  __syncthreads();
   float m[RMAX];
 #pragma unroll
   for (int q = 0; q < RMAX; ++q) m[q] = 0.f;
@@ -784,8 +800,7 @@ __global__ void k_cgt_p(float2* p, const float2* __restrict__ r, size_t ne, int 
         const size_t e = t * R + q;
         float2 pv = p[e];
         if (!ctl->done[q]) {
-          const double ro = ctl->rr[par][q], rn = ctl->rr[par ^ 1][q];
-          const float beta = (float)(ro > 0 ? rn / ro : 0.0);
+          const float beta = s_be[q];
           const float2 rv = r[e];
           pv.x = rv.x + beta * pv.x;
           pv.y = rv.y + beta * pv.y;
@@ -846,18 +861,25 @@ __global__ void __cluster_dims__(CS_CTAS, 1, 1) __launch_bounds__(CS_THREADS)
   if (ctl->all_done) return;   // written by CTA 0 behind the last barrier only
   __shared__ float shi[CS_THREADS], slo[CS_THREADS];
   __shared__ unsigned sxm[RMAX];
+  __shared__ double s_rn[RMAX];
+  __shared__ float s_al[RMAX], s_be[RMAX];
   const int cta = blockIdx.x, tid = threadIdx.x, gid = cta * CS_THREADS + tid;
   const int stride = CS_CTAS * CS_THREADS / Rp * Rp;    // whole groups of Rp: a thread keeps its right-hand side
   const int q = gid % Rp, KG = Kp / 8, N = Vc * KG * Rp;
   const bool live = gid < stride && q < R;
   const bool run = live && !ctl->done[q];
   if (tid < RMAX) sxm[tid] = 0u;
-  const double ro = live ? ctl->rr[par][q] : 0.0;
+  // FP64 divisions and sums once per right-hand side and CTA: by every thread they
+  // were most of the kernel (FP64 does two lanes per clock and SM)
+  if (tid < R) {
+    const double pap = ctl->pAp[tid];
+    s_al[tid] = (float)(pap > 0 ? ctl->rr[par][tid] / pap : 0.0);
+  }
+  __syncthreads();
   // x += alpha p, r -= alpha w, |r|^2
   float s = 0.f, e = 0.f;
   if (live) {
-    const double pap = ctl->pAp[q];
-    const float al = (float)(pap > 0 ? ro / pap : 0.0);
+    const float al = s_al[q];
     for (int j = gid; j < N; j += stride) {
       const int it = j / Rp, a = it / KG, k0 = 8 * (it % KG), kc = min(8, n - k0);
       const size_t o0 = ((size_t)a * n + k0) * R + q;
@@ -892,10 +914,7 @@ __global__ void __cluster_dims__(CS_CTAS, 1, 1) __launch_bounds__(CS_THREADS)
           }
 #pragma unroll
           for (int c = 0; c < 2; ++c) {
-            const float v = c ? rv[k].y : rv[k].x, sq = __fmul_rn(v, v), d = __fmaf_rn(v, v, -sq);
-            float u;
-            two_sum(s, sq, s, u);
-            e = __fadd_rn(e, __fadd_rn(u, d));
+            add_square(s, e, c ? rv[k].y : rv[k].x);
           }
         }
       }
@@ -908,20 +927,37 @@ __global__ void __cluster_dims__(CS_CTAS, 1, 1) __launch_bounds__(CS_THREADS)
     // warp w sums right-hand side w over the CTA's threads
     const int wq = tid >> 5;
     if (wq < R) {
-      double t = 0.0;
-      for (int i = tid & 31; i < CS_THREADS; i += 32)
-        if ((cta * CS_THREADS + i) % Rp == wq) t += (double)shi[i] + (double)slo[i];
+      float h = 0.f, l = 0.f;
+      int i = (wq - cta * CS_THREADS % Rp + Rp) % Rp;      // the CTA's first thread of this right-hand side
+      for (i += (tid & 31) * Rp; i < CS_THREADS; i += 32 * Rp) {
+        float u, v;
+        two_sum(h, shi[i], u, v);
+        h = u;
+        l = __fadd_rn(l, __fadd_rn(v, slo[i]));
+      }
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(FULL_MASK, t, o);
-      if ((tid & 31) == 0) sc->rr[cta][wq] = t;
+      for (int o = 16; o > 0; o >>= 1) {
+        const float oh = __shfl_xor_sync(FULL_MASK, h, o), ol = __shfl_xor_sync(FULL_MASK, l, o);
+        float u, v;
+        two_sum(h, oh, u, v);
+        h = u;
+        l = __fadd_rn(v, __fadd_rn(l, ol));
+      }
+      if ((tid & 31) == 0) sc->rr[cta][wq] = widen(h) + widen(l);
     }
   }
   cluster_sync();
   // p = r + beta p, max |p|
-  double rn = 0.0;
+  if (tid < R) {
+    double rn = 0.0;
+    for (int c = 0; c < CS_CTAS; ++c) rn += __ldcg(&sc->rr[c][tid]);
+    const double ro = ctl->rr[par][tid];
+    s_rn[tid] = rn;
+    s_be[tid] = (float)(ro > 0 ? rn / ro : 0.0);
+  }
+  __syncthreads();
   if (live) {
-    for (int c = 0; c < CS_CTAS; ++c) rn += __ldcg(&sc->rr[c][q]);
-    const float be = (float)(ro > 0 ? rn / ro : 0.0);
+    const float be = s_be[q];
     float m = 0.f;
     for (int j = gid; j < N; j += stride) {
       const int it = j / Rp, a = it / KG, k0 = 8 * (it % KG), kc = min(8, n - k0);
@@ -981,7 +1017,7 @@ __global__ void __cluster_dims__(CS_CTAS, 1, 1) __launch_bounds__(CS_THREADS)
   }
   // bookkeeping (nobody reads it in this launch any more)
   if (gid < R) {
-    ctl->rr[par ^ 1][gid] = rn;
+    ctl->rr[par ^ 1][gid] = s_rn[gid];
     xmax[gid] = xm;
   }
   if (cta == 0) {

@@ -278,4 +278,30 @@ __device__ bool grid_reduce(double (&v)[NV], const Reduction& red, int active = 
   return true;
 }
 
+// grid_reduce of per-thread double-float pairs: warps sum by TwoSum on the FP32
+// pipes and only the warp totals are added in FP64, whose pipe (two lanes per clock
+// and SM) otherwise bounds short vector kernels
+template <int NV>
+__device__ __forceinline__ bool grid_reduce_pairs(float (&hi)[NV], float (&lo)[NV], const Reduction& red,
+                                                  int active = RED_RHS) {
+  double v[NV];
+#pragma unroll
+  for (int i = 0; i < NV; ++i) {
+    v[i] = 0.0;
+    if (red_active<NV>(i, active)) {
+      float h = hi[i], l = lo[i];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        const float oh = __shfl_xor_sync(FULL_MASK, h, o), ol = __shfl_xor_sync(FULL_MASK, l, o);
+        float s, e;
+        two_sum(h, oh, s, e);
+        h = s;
+        l = __fadd_rn(e, __fadd_rn(l, ol));
+      }
+      v[i] = widen(h) + widen(l);
+    }
+  }
+  return grid_reduce<NV, true>(v, red, active);
+}
+
 }  // namespace hdcg

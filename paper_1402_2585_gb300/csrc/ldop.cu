@@ -396,6 +396,12 @@ __global__ void k_ad1_update(float2* x, float2* r, const float2* __restrict__ p,
   if (t == 0 && xmax)
     for (int q = 0; q < RMAX; ++q) xmax[q] = 0u;
   const size_t nc = ne * R;
+  __shared__ float s_al[RMAX];
+  if (threadIdx.x < R) {
+    const double pap = ctl->pAp[threadIdx.x];
+    s_al[threadIdx.x] = (float)(pap != 0.0 ? ctl->dots[par][threadIdx.x] / pap : 0.0);
+  }
+  __syncthreads();
   double v[RMAX];
 #pragma unroll
   for (int q = 0; q < RMAX; ++q) v[q] = 0.0;
@@ -406,8 +412,7 @@ __global__ void k_ad1_update(float2* x, float2* r, const float2* __restrict__ p,
         const size_t o = t * R + q;
         float2 rv = r[o];
         if (!ctl->done[q]) {
-          const double pap = ctl->pAp[q];
-          const float al = (float)(pap != 0.0 ? ctl->dots[par][q] / pap : 0.0);
+          const float al = s_al[q];
           float2 wv = w[o];
           for (int g = 1; g < ngroups; ++g) {
             wv.x += w[(size_t)g * nc + o].x;
@@ -446,6 +451,13 @@ __global__ void k_ad1_p(float2* p, const float2* __restrict__ y, size_t ne, int 
                         int first, unsigned* xmax) {
   if (ctl->all_done) return;
   const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  __shared__ float s_be[RMAX];
+  if (threadIdx.x < R) {
+    const int q = threadIdx.x;
+    const double ry_old = first ? 0.0 : ctl->dots[par ^ 1][q];
+    s_be[q] = (float)(ry_old != 0.0 ? (ctl->dots[par][q] - ctl->dots[par][RMAX + q]) / ry_old : 0.0);
+  }
+  __syncthreads();
   float m[RMAX];
 #pragma unroll
   for (int q = 0; q < RMAX; ++q) m[q] = 0.f;
@@ -457,11 +469,7 @@ __global__ void k_ad1_p(float2* p, const float2* __restrict__ y, size_t ne, int 
         // first: p is work memory nobody wrote yet (0 x NaN would survive beta = 0)
         float2 pv = first ? make_float2(0.f, 0.f) : p[o];
         if (!ctl->done[q]) {
-          float beta = 0.f;
-          if (!first) {
-            const double ry_old = ctl->dots[par ^ 1][q];
-            beta = (float)(ry_old != 0.0 ? (ctl->dots[par][q] - ctl->dots[par][RMAX + q]) / ry_old : 0.0);
-          }
+          const float beta = s_be[q];
           const float2 yv = y[o];
           pv.x = yv.x + beta * pv.x;
           pv.y = yv.y + beta * pv.y;

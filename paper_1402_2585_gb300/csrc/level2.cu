@@ -666,6 +666,13 @@ __global__ void k_l1_p(float2* p, const float2* __restrict__ y, size_t ne, int R
   if (ctl->all_done) return;
   const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t < RMAX) ctl->xm[1][t] = 0u;
+  __shared__ float s_be[RMAX];
+  if (threadIdx.x < R) {
+    const int q = threadIdx.x;
+    const double ro = first ? 0.0 : ctl->ry[par][q];
+    s_be[q] = (float)(ro != 0.0 ? (ctl->ry[par ^ 1][q] - ctl->ryo[q]) / ro : 0.0);
+  }
+  __syncthreads();
   float m[RMAX];
 #pragma unroll
   for (int q = 0; q < RMAX; ++q) m[q] = 0.f;
@@ -677,11 +684,7 @@ __global__ void k_l1_p(float2* p, const float2* __restrict__ y, size_t ne, int R
         // first: p is work memory nobody wrote yet (0 x NaN would survive beta = 0)
         float2 pv = first ? make_float2(0.f, 0.f) : p[o];
         if (!ctl->done[q]) {
-          float beta = 0.f;
-          if (!first) {
-            const double ro = ctl->ry[par][q];
-            beta = (float)(ro != 0.0 ? (ctl->ry[par ^ 1][q] - ctl->ryo[q]) / ro : 0.0);
-          }
+          const float beta = s_be[q];
           const float2 yv = y[o];
           pv.x = yv.x + beta * pv.x;
           pv.y = yv.y + beta * pv.y;
@@ -702,6 +705,12 @@ __global__ void k_l1_update(float2* x, float2* r, const float2* __restrict__ p, 
   if (ctl->all_done) return;
   const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t < RMAX) ctl->xm[0][t] = 0u;
+  __shared__ float s_al[RMAX];
+  if (threadIdx.x < R) {
+    const double pap = ctl->pAp[threadIdx.x];
+    s_al[threadIdx.x] = pap > 0.0 ? (float)(ctl->ry[par][threadIdx.x] / pap) : 0.f;
+  }
+  __syncthreads();
   double v[2 * RMAX];
   float m[RMAX];
 #pragma unroll
@@ -717,8 +726,7 @@ __global__ void k_l1_update(float2* x, float2* r, const float2* __restrict__ p, 
         // (p, A p) <= 0 (a rounded operator that is not positive definite at the
         // bottom of its spectrum) ends the right-hand side's iteration unchanged
         if (!ctl->done[q] && ctl->pAp[q] > 0.0) {
-          const double pap = ctl->pAp[q];
-          const float al = (float)(ctl->ry[par][q] / pap);
+          const float al = s_al[q];
           const float2 pv = p[o], wv = w[o];
           float2 xv = x[o];
           xv.x += al * pv.x;
