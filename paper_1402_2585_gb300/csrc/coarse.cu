@@ -1357,7 +1357,7 @@ static int coarse_cg_t(Ctx& c, Coarse& A, const void* rhs, void* sol, double tol
   c.launches += 2;
   int queued = 0;
   int batch = std::max(1, A.last_iters);
-  CCtl h{};
+  CCtl& h = *c.pinned.at<CCtl>(4096);
   while (true) {
     for (int b = 0; b < batch && queued < maxiter; ++b, ++queued) {
       const int par = queued & 1;
@@ -2016,7 +2016,7 @@ static int coarse_cg_multi_t(Ctx& c, Coarse& A, int R, const void* rhs, void* so
   c.launches += 2;
   int queued = 0;
   int batch = std::max(1, A.last_iters);
-  CCtlM h{};
+  CCtlM& h = *c.pinned.at<CCtlM>(4096);
   while (true) {
     for (int bq = 0; bq < batch && queued < maxiter; ++bq, ++queued) {
       const int par = queued & 1;

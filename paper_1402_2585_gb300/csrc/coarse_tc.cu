@@ -562,9 +562,10 @@ void coarse_tc_prepare(Ctx& c, Coarse& A) {
 }
 
 void coarse_tc_check(Ctx& c, Coarse& A) {
-  unsigned err = 0;
-  HDCG_CUDA(cudaMemcpyAsync(&err, &A.tcs.as<TcState>()->err, sizeof(unsigned), cudaMemcpyDeviceToHost, c.stream));
+  unsigned* flags = c.pinned.at<unsigned>(8064);
+  HDCG_CUDA(cudaMemcpyAsync(flags, &A.tcs.as<TcState>()->err, sizeof(unsigned), cudaMemcpyDeviceToHost, c.stream));
   HDCG_CUDA(cudaStreamSynchronize(c.stream));
+  const unsigned err = *flags;
   if (err) {
     HDCG_CUDA(cudaMemsetAsync(A.tcs.p, 0, sizeof(unsigned), c.stream));
     throw Error{HDCG_ERR_TIMEOUT, "tensor-core coarse apply: a pipeline wait expired (flags " +
@@ -1094,7 +1095,7 @@ int coarse_cg_tc(Ctx& c, Coarse& A, int R, const void* rhs, void* sol, double to
                                       (uintptr_t)shift_bits};
   int queued = 0;
   int batch = std::max(2, A.last_iters);
-  CCtlT h{};
+  CCtlT& h = *c.pinned.at<CCtlT>(4096);
   while (true) {
     for (int bq = 0; bq < batch && queued < maxiter; bq += 2, queued += 2) {
       if (queued == 0) {

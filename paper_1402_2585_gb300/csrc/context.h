@@ -80,6 +80,31 @@ struct DevMem {
   template <typename T> T* as() const { return reinterpret_cast<T*>(p); }
 };
 
+// page-locked host memory for the scalars and control blocks that a solver loop
+// reads back: copies into it are queued and waited for once (a copy into pageable
+// memory waits for the stream by itself, every one of them)
+struct PinnedMem {
+  void* p = nullptr;
+  static constexpr size_t bytes = 8192;
+  PinnedMem() = default;
+  PinnedMem(const PinnedMem&) = delete;
+  PinnedMem& operator=(const PinnedMem&) = delete;
+  ~PinnedMem() {
+    if (p) cudaFreeHost(p);
+  }
+  template <typename T> T* at(size_t offset = 0) {
+    if (!p) {
+      const cudaError_t e = cudaMallocHost(&p, bytes);
+      if (e != cudaSuccess) {
+        p = nullptr;
+        (void)cudaGetLastError();
+        throw Error{HDCG_ERR_OOM, "page-locked host memory for the solver's scalars"};
+      }
+    }
+    return reinterpret_cast<T*>(static_cast<char*>(p) + offset);
+  }
+};
+
 // a fine odd/even field in the internal chunked layout
 struct FieldRef {
   uint4* p;
@@ -134,6 +159,7 @@ struct Ctx {
   int hop_force = -1;            // >= 0: every hop launch uses this variant (hdcg_set_hop_variant)
   int tc_force = 0;              // 1, 2: the tensor-core stencil's CTAs per SM (hdcg_set_coarse_tc_shape)
   DevMem red_partials, red_ticket, scalars;
+  PinnedMem pinned;              // scalars at 0, a solver's control block at 4096, error flags at 8064
   DevMem canon_in, canon_out;  // canonical <-> internal staging
   // coarse vectors of the calls on canonical coarse vectors: kept by the handle
   // (cudaMalloc and cudaFree cost more than a small coarse apply), two because a

@@ -812,7 +812,7 @@ int coarse_adef1(Ctx& c, Coarse& A, int R, const void* rhs, void* sol, double to
       (uintptr_t)ne, (uintptr_t)tc, (uintptr_t)maxiter};
   int queued = 0;
   int batch = std::max(2, A.last_iters);
-  CCtlD h{};
+  CCtlD& h = *c.pinned.at<CCtlD>(4096);
   while (true) {
     for (int bq = 0; bq < batch && queued < maxiter; bq += 2, queued += 2) {
       if (queued == 0) {

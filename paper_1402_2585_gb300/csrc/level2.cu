@@ -1172,7 +1172,7 @@ int level1_solve(Ctx& c, Coarse& A, int R, const void* rhs, void* sol, double to
                                       (uintptr_t)A.qt.work.p, (uintptr_t)A.qt.A9.p};
   int queued = 0;
   int batch = std::max(2, L.last_iters);
-  CtlL2 h{};
+  CtlL2& h = *c.pinned.at<CtlL2>(4096);
   HDCG_CUDA(cudaMemcpyAsync(&h, ctl, sizeof(CtlL2), cudaMemcpyDeviceToHost, c.stream));
   HDCG_CUDA(cudaStreamSynchronize(c.stream));
   while (!h.all_done) {

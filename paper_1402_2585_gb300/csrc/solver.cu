@@ -49,9 +49,18 @@ static double* dsc(Ctx& c, int slot) { return c.scalars.as<double>() + slot * RM
 
 // read scalar slots [slot, slot + n) of right-hand side 0
 static void read_scalars(Ctx& c, int slot, int n, double* h) {
-  for (int i = 0; i < n; ++i)
-    HDCG_CUDA(cudaMemcpyAsync(h + i, dsc(c, slot + i), sizeof(double), cudaMemcpyDeviceToHost, c.stream));
+  double* v = c.pinned.at<double>();
+  HDCG_CUDA(cudaMemcpyAsync(v, dsc(c, slot), ((n - 1) * RMAX + 1) * sizeof(double), cudaMemcpyDeviceToHost, c.stream));
   HDCG_CUDA(cudaStreamSynchronize(c.stream));
+  for (int i = 0; i < n; ++i) h[i] = v[i * RMAX];
+}
+
+// the same for every right-hand side: slot + i into h[i]
+static void read_scalars_multi(Ctx& c, int slot, int n, int R, double* const* h) {
+  double* v = c.pinned.at<double>();
+  HDCG_CUDA(cudaMemcpyAsync(v, dsc(c, slot), n * RMAX * sizeof(double), cudaMemcpyDeviceToHost, c.stream));
+  HDCG_CUDA(cudaStreamSynchronize(c.stream));
+  for (int i = 0; i < n; ++i) std::memcpy(h[i], v + i * RMAX, R * sizeof(double));
 }
 
 static void copy_scalar(Ctx& c, int dst, int src) {
@@ -530,9 +539,8 @@ static int solve_batch(Ctx& c, const uint4* b64, uint4* x64, int R, double tol, 
     st->n_mdagm_outer += R;
     ++it;
     double pw[RMAX];
-    HDCG_CUDA(cudaMemcpyAsync(pw, dsc(c, D_PW), R * sizeof(double), cudaMemcpyDeviceToHost, c.stream));
-    HDCG_CUDA(cudaMemcpyAsync(rr, dsc(c, D_RR), R * sizeof(double), cudaMemcpyDeviceToHost, c.stream));
-    HDCG_CUDA(cudaStreamSynchronize(c.stream));
+    double* const both[2] = {pw, rr};
+    read_scalars_multi(c, D_PW, 2, R, both);
     bool need = it >= prm.maxiter;
     for (int k = 0; k < R; ++k) {
       if (!mask[k]) continue;
