@@ -588,19 +588,15 @@ double mean_diag(Ctx& c, const Coarse& A) {
   return h;
 }
 
-// Y = A X for R <= 16 FP32 vectors [e][r] (tensor cores for FP16 A)
+// Y = A X for R <= 16 FP32 vectors [e][r], in FP32 multiply-adds whatever the
+// solver's product uses. The Ritz values are quotients with these products, and
+// an error e of theirs moves a value by x^dag e. The tensor cores' sums are
+// truncated: x^dag e is 1.4e-7 on average there (3^4 sites, Nvec 8, |A| = 2.8)
+// against 5e-9 here, which is 1e-5 of a lowest value of 0.01. It is nvec / 16
+// products of a setup that solves nvec systems several times over.
 void apply_batch(Ctx& c, Coarse& A, int R, const float2* X, float2* Y, DevMem& part, DevMem& dots) {
   const size_t ne = A.Vc * A.nvec;
   dots.ensure(RMAX * sizeof(double));
-  if (coarse_tc_supported(A)) {
-    coarse_tc_prepare(c, A);
-    unsigned* xmax = A.tcs.as<TcState>()->xmax;
-    coarse_tc_max(c, X, ne, R, xmax);
-    coarse_tc_to_b(c, A, R, X, xmax, nullptr);
-    coarse_tc_apply(c, A, R, X, Y, xmax, nullptr, nullptr, 0.0);
-    coarse_tc_check(c, A);
-    return;
-  }
   part.ensure((size_t)4 * ne * R * sizeof(float2));
   const int ng = coarse_apply_partials(c, A, R, X, part.as<float2>(), nullptr, dots.as<double>());
   k_sum_parts<<<blocks(ne * R), 256, 0, c.stream>>>(part.as<float2>(), ne * R, ng, Y);
