@@ -539,14 +539,18 @@ __global__ void __launch_bounds__(256) k_restrict(const uint4* __restrict__ phi,
         Rp p[P];
         unpack(Sp{}, raw[k], p);
 #pragma unroll
-        for (int r = 0; r < RB; ++r)
+        for (int r = 0; r < RB; ++r) {
+          T re = 0, im = 0;   // a granule first: a quarter of the long sums' roundings
 #pragma unroll
           for (int e = 0; e < P; e += 2) {
-            acc[k][r][0] += (T)p[e] * vv[r][e];
-            acc[k][r][0] += (T)p[e + 1] * vv[r][e + 1];
-            acc[k][r][1] += (T)p[e] * vv[r][e + 1];
-            acc[k][r][1] -= (T)p[e + 1] * vv[r][e];
+            re += (T)p[e] * vv[r][e];
+            re += (T)p[e + 1] * vv[r][e + 1];
+            im += (T)p[e] * vv[r][e + 1];
+            im -= (T)p[e + 1] * vv[r][e];
           }
+          acc[k][r][0] += re;
+          acc[k][r][1] += im;
+        }
       }
     }
     double s[32];
