@@ -496,6 +496,15 @@ __device__ __forceinline__ double warp_scatter_sum(double (&v)[32]) {
 // site with sums of 32 doubles per warp by butterflies: 2408 us for 24^3 x 48 x 16,
 // 32 FP16 vectors, 8.4 GB; both kernels of this file together now take 2.6 ms of
 // P R at that size, of 3.6.)
+// a += x, the rounding kept in l (Knuth's TwoSum). Plain FP32 sums over a block gave
+// 1.8e-7 of error on 16^4 x 16 (21 vectors, both projections, 512 us); so 1.3e-7, 616 us
+template <typename T>
+__device__ __forceinline__ void add_keep(T& a, T& l, T x) {
+  const T s = a + x, bb = s - a;
+  l += (a - (s - bb)) + (x - bb);
+  a = s;
+}
+
 template <typename Sp, typename Sv, typename Rc, int KC, int RB>
 __global__ void __launch_bounds__(256) k_restrict(const uint4* __restrict__ phi, size_t pstride, int nvec,
                                                   const uint4* __restrict__ v, size_t vstride, int R, BlockArgs ba,
@@ -511,11 +520,12 @@ __global__ void __launch_bounds__(256) k_restrict(const uint4* __restrict__ phi,
   const int ng = ba.spb * ba.Ls * C;
   for (int r0 = 0; r0 < R; r0 += RB) {
     const int rb = min(RB, R - r0);
-    T acc[KC][RB][2];
+    constexpr bool KEEP = sizeof(T) == 4;
+    T acc[KC][RB][2], low[KC][RB][2];
 #pragma unroll
     for (int k = 0; k < KC; ++k)
 #pragma unroll
-      for (int r = 0; r < RB; ++r) acc[k][r][0] = acc[k][r][1] = 0;
+      for (int r = 0; r < RB; ++r) acc[k][r][0] = acc[k][r][1] = low[k][r][0] = low[k][r][1] = 0;
     for (int i = threadIdx.x; i < ng; i += 256) {
       // chunk-major storage: consecutive threads take consecutive sites of a chunk
       const int ch = C == 3 ? i % 3 : i / (ba.spb * ba.Ls), g = C == 3 ? i / 3 : i % (ba.spb * ba.Ls);
@@ -548,14 +558,19 @@ __global__ void __launch_bounds__(256) k_restrict(const uint4* __restrict__ phi,
             im += (T)p[e] * vv[r][e + 1];
             im -= (T)p[e + 1] * vv[r][e];
           }
-          acc[k][r][0] += re;
-          acc[k][r][1] += im;
+          if constexpr (KEEP) {
+            add_keep(acc[k][r][0], low[k][r][0], re);
+            add_keep(acc[k][r][1], low[k][r][1], im);
+          } else {
+            acc[k][r][0] += re;
+            acc[k][r][1] += im;
+          }
         }
       }
     }
     double s[32];
 #pragma unroll
-    for (int q = 0; q < 32; ++q) s[q] = widen(acc[(q / 2) / RB][(q / 2) % RB][q & 1]);
+    for (int q = 0; q < 32; ++q) s[q] = widen(acc[(q / 2) / RB][(q / 2) % RB][q & 1] + low[(q / 2) / RB][(q / 2) % RB][q & 1]);
     const double total = warp_scatter_sum(s);
     __syncthreads();
     part[threadIdx.x >> 5][threadIdx.x & 31] = total;
