@@ -488,14 +488,6 @@ __device__ __forceinline__ double warp_scatter_sum(double (&v)[32]) {
   return v[0];
 }
 
-// c[b][k][r] = <phi_k^b, v_r>: one CTA per block (x) and group of KC vectors (y).  A thread owns granules of the
-// subspace's layout: RB fields' values of a granule stay in registers while the KC
-// vectors stream by in 16-byte loads, so lanes read consecutive granules in every
-// layout.  Thread sums are FP32 (FP64 with FP64 operands) over its granules, the
-// sums over threads FP64.  Bound by the stream of the vectors.  (One thread per
-// site with sums of 32 doubles per warp by butterflies: 2408 us for 24^3 x 48 x 16,
-// 32 FP16 vectors, 8.4 GB; both kernels of this file together now take 2.6 ms of
-// P R at that size, of 3.6.)
 // a += x, the rounding kept in l (Knuth's TwoSum). Plain FP32 sums over a block gave
 // 1.8e-7 of error on 16^4 x 16 (21 vectors, both projections, 512 us); so 1.3e-7, 616 us
 template <typename T>
@@ -505,6 +497,14 @@ __device__ __forceinline__ void add_keep(T& a, T& l, T x) {
   a = s;
 }
 
+// c[b][k][r] = <phi_k^b, v_r>: one CTA per block (x) and group of KC vectors (y).  A thread owns granules of the
+// subspace's layout: RB fields' values of a granule stay in registers while the KC
+// vectors stream by in 16-byte loads, so lanes read consecutive granules in every
+// layout.  Thread sums are FP32 (FP64 with FP64 operands) over its granules, the
+// sums over threads FP64.  Bound by the stream of the vectors.  (One thread per
+// site with sums of 32 doubles per warp by butterflies: 2408 us for 24^3 x 48 x 16,
+// 32 FP16 vectors, 8.4 GB; both kernels of this file together now take 2.6 ms of
+// P R at that size, of 3.6.)
 template <typename Sp, typename Sv, typename Rc, int KC, int RB>
 __global__ void __launch_bounds__(256) k_restrict(const uint4* __restrict__ phi, size_t pstride, int nvec,
                                                   const uint4* __restrict__ v, size_t vstride, int R, BlockArgs ba,
