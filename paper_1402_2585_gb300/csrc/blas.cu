@@ -5,8 +5,6 @@
 // hence different chunking) line up.  Every reduction accumulates in FP64
 // (per-thread FP32/FP64 partial over 24 reals, then FP64 warp / block / grid
 // sums in a fixed order: two runs give bit-identical results).
-#include <type_traits>
-
 #include "blas.cuh"
 
 namespace hdcg {
@@ -256,19 +254,6 @@ void zero_field(Ctx& c, uint4* f, int prec, size_t nf) {
 // ---------------------------------------------------------------------------
 // reductions
 // ---------------------------------------------------------------------------
-// the NV partial sums of a thread into the grid reduction: FP32 partials through
-// double-float warp sums, FP64 ones in FP64
-template <int NV, typename R>
-__device__ __forceinline__ void reduce_partials(R (&s)[NV], const Reduction& red) {
-  if constexpr (std::is_same<R, float>::value) {
-    float lo[NV];
-#pragma unroll
-    for (int i = 0; i < NV; ++i) lo[i] = 0.f;
-    grid_reduce_pairs<NV>(s, lo, red);
-  } else {
-    grid_reduce<NV>(s, red);
-  }
-}
 template <typename S>
 __global__ void k_norm2(const uint4* __restrict__ a, size_t n5, Reduction red, size_t fstride) {
   using R = typename Store<S>::real;
@@ -283,7 +268,7 @@ __global__ void k_norm2(const uint4* __restrict__ a, size_t n5, Reduction red, s
     for (int i = 0; i < 24; ++i) s += x[i] * x[i];
     v[0] = s;
   }
-  reduce_partials<1>(v, red);
+  grid_reduce_shared<1>(v, red);
 }
 
 template <typename S>
@@ -415,7 +400,7 @@ __global__ void k_update_p(uint4* p, const uint4* __restrict__ y, size_t n5, Sca
     store_spinor<S, R>(p, t, n5, pv);
     v[0] = s;
   }
-  if (do_red) reduce_partials<1>(v, red);
+  if (do_red) grid_reduce_shared<1>(v, red);
 }
 
 // res[0] = Re<a, b>, res[1] = Re<a, c> (c may be null)
@@ -445,7 +430,7 @@ __global__ void k_redot2(const uint4* __restrict__ a, const uint4* __restrict__ 
     v[0] = s0;
     v[1] = s1;
   }
-  reduce_partials<2>(v, red);
+  grid_reduce_shared<2>(v, red);
 }
 
 // hi += lo ; lo = 0

@@ -752,9 +752,9 @@ __global__ void k_cgt_update(float2* x, float2* r, const float2* __restrict__ p,
     s_al[threadIdx.x] = (float)(pap > 0 ? ctl->rr[par][threadIdx.x] / pap : 0.0);
   }
   __syncthreads();
-  float hi[RMAX], lo[RMAX];
+  double v[RMAX];
 #pragma unroll
-  for (int q = 0; q < RMAX; ++q) hi[q] = lo[q] = 0.f;
+  for (int q = 0; q < RMAX; ++q) v[q] = 0.0;
   if (t < ne) {
 #pragma unroll
     for (int q = 0; q < RMAX; ++q) {
@@ -772,12 +772,12 @@ __global__ void k_cgt_update(float2* x, float2* r, const float2* __restrict__ p,
           x[e] = xv;
           r[e] = rv;
         }
-        add_square(hi[q], lo[q], rv.x);
-        add_square(hi[q], lo[q], rv.y);
+        const double re = widen(rv.x), im = widen(rv.y);
+        v[q] = fma(re, re, im * im);
       }
     }
   }
-  grid_reduce_pairs<RMAX>(hi, lo, red, R);
+  grid_reduce_shared<RMAX>(v, red, R);
 }
 
 // p = r + beta p for the right-hand sides still running; max|p| of every right-hand side
@@ -845,7 +845,7 @@ __global__ void k_cgt_check(CCtlT* ctl, int R, int par, int maxiter) {
 // With the split couplings (78 us a product on 128 of 152 SMs before, for 95 MB)
 // the batched solve of four sources on 16^4 x 16 went from 217 to 202 ms.
 // A thread owns the same (site, eight coefficients, right-hand side) items in every
-// phase.  |r|^2 sums by TwoProd and TwoSum (about 48 bits), CTAs in FP64.
+// phase.  |r|^2 in FP64, squares and sums: entries of FP32's whole range.
 // ---------------------------------------------------------------------------------
 constexpr int CS_CTAS = 8, CS_THREADS = 512, CS_ITEMS = 4;   // at most CS_ITEMS items a thread
 struct CgStepScratch {
@@ -861,7 +861,7 @@ __global__ void __cluster_dims__(CS_CTAS, 1, 1) __launch_bounds__(CS_THREADS)
     k_cgt_step(float2* x, float2* r, float2* p, const float2* w, int nsplit, size_t part, int Vc, int n, int R, int Rp,
                int Kp, char* xtc, CCtlT* ctl, CgStepScratch* sc, int par, int maxiter, unsigned* xmax) {
   if (ctl->all_done) return;   // written by CTA 0 behind the last barrier only
-  __shared__ float shi[CS_THREADS], slo[CS_THREADS];
+  __shared__ double srr[CS_THREADS];
   __shared__ unsigned sxm[RMAX];
   __shared__ double s_rn[RMAX];
   __shared__ float s_al[RMAX], s_be[RMAX];
@@ -879,7 +879,7 @@ __global__ void __cluster_dims__(CS_CTAS, 1, 1) __launch_bounds__(CS_THREADS)
   }
   __syncthreads();
   // x += alpha p, r -= alpha w, |r|^2
-  float s = 0.f, e = 0.f;
+  double s = 0.0;
   if (live) {
     const float al = s_al[q];
     for (int j = gid; j < N; j += stride) {
@@ -914,38 +914,25 @@ __global__ void __cluster_dims__(CS_CTAS, 1, 1) __launch_bounds__(CS_THREADS)
             x[o] = xv[k];
             r[o] = rv[k];
           }
-#pragma unroll
-          for (int c = 0; c < 2; ++c) {
-            add_square(s, e, c ? rv[k].y : rv[k].x);
-          }
+          const double re = widen(rv[k].x), im = widen(rv[k].y);
+          s = fma(re, re, s);
+          s = fma(im, im, s);
         }
       }
     }
   }
-  shi[tid] = s;
-  slo[tid] = e;
+  srr[tid] = s;
   __syncthreads();
   {
     // warp w sums right-hand side w over the CTA's threads
     const int wq = tid >> 5;
     if (wq < R) {
-      float h = 0.f, l = 0.f;
+      double v = 0.0;
       int i = (wq - cta * CS_THREADS % Rp + Rp) % Rp;      // the CTA's first thread of this right-hand side
-      for (i += (tid & 31) * Rp; i < CS_THREADS; i += 32 * Rp) {
-        float u, v;
-        two_sum(h, shi[i], u, v);
-        h = u;
-        l = __fadd_rn(l, __fadd_rn(v, slo[i]));
-      }
+      for (i += (tid & 31) * Rp; i < CS_THREADS; i += 32 * Rp) v += srr[i];
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const float oh = __shfl_xor_sync(FULL_MASK, h, o), ol = __shfl_xor_sync(FULL_MASK, l, o);
-        float u, v;
-        two_sum(h, oh, u, v);
-        h = u;
-        l = __fadd_rn(v, __fadd_rn(l, ol));
-      }
-      if ((tid & 31) == 0) sc->rr[cta][wq] = widen(h) + widen(l);
+      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(FULL_MASK, v, o);
+      if ((tid & 31) == 0) sc->rr[cta][wq] = v;
     }
   }
   cluster_sync();

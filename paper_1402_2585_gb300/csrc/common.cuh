@@ -228,11 +228,10 @@ struct Reduction {
   int result_stride;    // doubles between the results of consecutive right-hand sides
 };
 
-// Returns true in every thread of the last block (after the totals are stored).
-// PRE: v already holds per-warp sums in lane 0 (see block_sum).
-template <int NV, bool PRE = false>
-__device__ bool grid_reduce(double (&v)[NV], const Reduction& red, int active = RED_RHS) {
-  block_sum<NV, PRE>(v, active);
+// The grid's part of a reduction: v holds the CTA's sums in thread 0.  Returns true
+// in every thread of the last block (after the totals are stored).
+template <int NV>
+__device__ bool grid_finish(double (&v)[NV], const Reduction& red, int active) {
   __shared__ bool last;
   const unsigned y = blockIdx.y;
   double* partials = red.partials + (size_t)NV * gridDim.x * y;
@@ -278,30 +277,41 @@ __device__ bool grid_reduce(double (&v)[NV], const Reduction& red, int active = 
   return true;
 }
 
-// grid_reduce of per-thread double-float pairs: warps sum by TwoSum on the FP32
-// pipes and only the warp totals are added in FP64, whose pipe (two lanes per clock
-// and SM) otherwise bounds short vector kernels
-template <int NV>
-__device__ __forceinline__ bool grid_reduce_pairs(float (&hi)[NV], float (&lo)[NV], const Reduction& red,
-                                                  int active = RED_RHS) {
+// Sums over the grid; PRE: v already holds per-warp sums in lane 0 (see block_sum).
+template <int NV, bool PRE = false>
+__device__ bool grid_reduce(double (&v)[NV], const Reduction& red, int active = RED_RHS) {
+  block_sum<NV, PRE>(v, active);
+  return grid_finish<NV>(v, red, active);
+}
+
+// grid_reduce of CTAs of at most 256 threads through shared memory: one warp sums a
+// value of all threads in FP64, 7 + 5 FP64 additions a lane.  Butterflies over every
+// warp (grid_reduce) are 40 for the same eight warps, and the FP64 pipe (two lanes per
+// clock and SM) bounds short vector kernels.  FP32 partials are exact in FP64, so the
+// sums have FP64's rounding and range whichever type the threads hold.
+template <int NV, typename T>
+__device__ __forceinline__ bool grid_reduce_shared(const T (&s)[NV], const Reduction& red, int active = RED_RHS) {
+  __shared__ T sh[NV][256];
+  __shared__ double total[NV];
+#pragma unroll
+  for (int i = 0; i < NV; ++i)
+    if (red_active<NV>(i, active)) sh[i][threadIdx.x] = s[i];
+  __syncthreads();
+  const int lane = threadIdx.x & 31;
+  for (int i = threadIdx.x >> 5; i < NV; i += (int)blockDim.x >> 5) {
+    double v = 0.0;
+    if (red_active<NV>(i, active)) {
+      for (int t = lane; t < (int)blockDim.x; t += 32) v += widen(sh[i][t]);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(FULL_MASK, v, o);
+    }
+    if (lane == 0) total[i] = v;
+  }
+  __syncthreads();
   double v[NV];
 #pragma unroll
-  for (int i = 0; i < NV; ++i) {
-    v[i] = 0.0;
-    if (red_active<NV>(i, active)) {
-      float h = hi[i], l = lo[i];
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const float oh = __shfl_xor_sync(FULL_MASK, h, o), ol = __shfl_xor_sync(FULL_MASK, l, o);
-        float s, e;
-        two_sum(h, oh, s, e);
-        h = s;
-        l = __fadd_rn(e, __fadd_rn(l, ol));
-      }
-      v[i] = widen(h) + widen(l);
-    }
-  }
-  return grid_reduce<NV, true>(v, red, active);
+  for (int i = 0; i < NV; ++i) v[i] = threadIdx.x == 0 ? total[i] : 0.0;
+  return grid_finish<NV>(v, red, active);
 }
 
 }  // namespace hdcg

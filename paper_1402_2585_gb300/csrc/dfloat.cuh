@@ -166,14 +166,6 @@ __device__ __forceinline__ float madd2(float a, float b, float c, float d) { ret
 __device__ __forceinline__ double madd2(double a, double b, double c, double d) { return a * b + c * d; }
 __device__ __forceinline__ dfl madd2(dfl a, dfl b, dfl c, dfl d) { return a * b + c * d; }
 
-// (s, e) += v v, about 48 bits, without the FP64 pipe
-__device__ __forceinline__ void add_square(float& s, float& e, float v) {
-  const float q = __fmul_rn(v, v), d = __fmaf_rn(v, v, -q);
-  float u;
-  two_sum(s, q, s, u);
-  e = __fadd_rn(e, __fadd_rn(u, d));
-}
-
 // lane shuffles of any compute type
 __device__ __forceinline__ float shfl_any(float v, int src, int width) {
   return __shfl_sync(0xffffffffu, v, src, width);

@@ -75,3 +75,46 @@ def kappa_tol(kappa, bar=1e-6, cap=1e-8):
     """Relative residual that bounds the solution error by bar / 2:
     |x - x*| / |x*| <= kappa |r| / |b|."""
     return min(cap, 0.5 * bar / kappa)
+
+
+def random_stencil(cd, n, rng):
+    """Hermitian nearest-neighbour operator [Vc][81][n][n] (complex64) on coarse
+    extents cd, spectrum within [0.4, 1.6], with the neighbour of every site per
+    offset and which offsets are stored (on an extent of 2 only the forward one,
+    on an extent of 1 none)."""
+    vc = int(np.prod(cd))
+    xs, r = [], np.arange(vc)
+    for L in cd:
+        xs.append(r % L)
+        r = r // L
+    nb, stored, mate = np.zeros((vc, 81), dtype=int), [], []
+    for l in range(81):
+        d = [l // 3 ** mu % 3 - 1 for mu in range(4)]
+        idx, mul, m = 0, 1, 0
+        for mu, L in enumerate(cd):
+            idx = idx + (xs[mu] + d[mu]) % L * mul
+            mul *= L
+            m += 3 ** mu * ((d[mu] if L == 2 else -d[mu]) + 1)
+        nb[:, l] = idx
+        mate.append(m)
+        stored.append(all(L >= 3 or (q >= 0 if L == 2 else q == 0) for q, L in zip(d, cd)))
+    A = np.zeros((vc, 81, n, n), dtype=np.complex64)
+    for l in range(81):
+        if not stored[l] or mate[l] < l:
+            continue
+        z = (rng.standard_normal((vc, n, n)) + 1j * rng.standard_normal((vc, n, n))) * (0.1 / np.sqrt(2 * n * sum(stored)))
+        if mate[l] == l:
+            z = 0.5 * (z + z[nb[:, l]].conj().transpose(0, 2, 1))
+        else:
+            A[nb[:, l], mate[l]] = z.conj().transpose(0, 2, 1)
+        A[:, l] = z
+    A[:, 40] += np.eye(n, dtype=np.complex64)
+    return A, nb, stored
+
+
+def apply_stencil(A, nb, stored, x):
+    y = np.zeros_like(x)
+    for l in range(81):
+        if stored[l]:
+            y += np.einsum("ajk,rak->raj", A[:, l].astype(np.complex128), x[:, nb[:, l]])
+    return y
