@@ -20,7 +20,6 @@
 #include <vector>
 
 #include "coarse.cuh"
-#include "mma.cuh"
 
 namespace hdcg {
 
@@ -503,8 +502,11 @@ __device__ __forceinline__ void add_keep(T& a, T& l, T x) {
 // layout.  Thread sums are FP32 (FP64 with FP64 operands) over its granules, the
 // sums over threads FP64.  Bound by the stream of the vectors.  (One thread per
 // site with sums of 32 doubles per warp by butterflies: 2408 us for 24^3 x 48 x 16,
-// 32 FP16 vectors, 8.4 GB; both kernels of this file together now take 2.6 ms of
-// P R at that size, of 3.6.)
+// 32 FP16 vectors, 8.4 GB; P R at that size took 4.6 ms then, 3.3 ms now.)
+// FP16 x FP16 on the tensor cores (mma.sync, exact products) takes 450 us less, but
+// its FP32 sums are truncated towards zero: over 512 products, flushed to a pair,
+// 6e-7 of error on random fields and 2.6e-6 on fields along the vectors, where these
+// sums have 6e-8 and 2e-8.
 template <typename Sp, typename Sv, typename Rc, int KC, int RB>
 __global__ void __launch_bounds__(256) k_restrict(const uint4* __restrict__ phi, size_t pstride, int nvec,
                                                   const uint4* __restrict__ v, size_t vstride, int R, BlockArgs ba,
@@ -588,97 +590,6 @@ __global__ void __launch_bounds__(256) k_restrict(const uint4* __restrict__ phi,
   }
 }
 
-// The same for 16-bit vectors and fields of one type, on the tensor cores: rows
-// are 16 subspace vectors, columns 8 right-hand sides, k the block's reals (exact
-// 16-bit products).  As in hop_tc.cuh k may be permuted: lane (g, t) loads granule
-// 4 i + t of vectors g and g + 8 and of field g, its four words are two k16 steps.
-// Re <phi, v> takes (v_re, v_im), Im (v_im, -v_re).  FP32 sums over 16 groups of
-// four granules (512 products) go to a double-float pair; the sums over warps are
-// FP64.  Reads each vector once for up to 16 right-hand sides.
-constexpr int RT_WARPS = 8, RT_FLUSH = 16;
-template <typename S, int NT>
-__global__ void __launch_bounds__(32 * RT_WARPS, 2) k_restrict_tc(const uint4* __restrict__ phi, size_t pstride,
-                                                                  int nvec, const uint4* __restrict__ v,
-                                                                  size_t vstride, int R, BlockArgs ba, float2* out) {
-  __shared__ double2 part[RT_WARPS][16][8];
-  const size_t b = blockIdx.x;
-  const int k0 = blockIdx.y * 16;
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
-  const int per = ba.Ls * 3;                     // granules of a 4D site
-  const int groups = ba.spb * per / 4;
-  const uint4* p0 = phi + (size_t)min(k0 + g, nvec - 1) * pstride;
-  const uint4* p1 = phi + (size_t)min(k0 + g + 8, nvec - 1) * pstride;
-  float hi[NT][2][4], lo[NT][2][4], acc[NT][2][4];
-#pragma unroll
-  for (int n = 0; n < NT; ++n)
-#pragma unroll
-    for (int h = 0; h < 2; ++h)
-#pragma unroll
-      for (int i = 0; i < 4; ++i) hi[n][h][i] = lo[n][h][i] = acc[n][h][i] = 0.f;
-  constexpr int U = 4;
-  int count = 0;
-  for (int i0 = w; i0 < groups; i0 += U * RT_WARPS) {
-    uint4 a0[U], a1[U], bv[U][NT];
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int i = i0 + u * RT_WARPS;
-      const int gr = 4 * min(i, groups - 1) + t;
-      const size_t at = (size_t)__ldg(ba.block_sites + b * ba.spb + gr / per) * per + gr % per;
-      a0[u] = __ldg(p0 + at);
-      a1[u] = __ldg(p1 + at);
-#pragma unroll
-      for (int n = 0; n < NT; ++n)
-        bv[u][n] = (8 * n + g < R && i < groups) ? __ldg(v + (size_t)(8 * n + g) * vstride + at) : make_uint4(0u, 0u, 0u, 0u);
-    }
-#pragma unroll
-    for (int u = 0; u < U; ++u)
-#pragma unroll
-      for (int n = 0; n < NT; ++n) {
-        const uint4 x = bv[u][n];
-        // (re, im) -> (im, -re)
-        auto turn = [](unsigned z) { return __byte_perm(z, 0u, 0x1032u) ^ 0x80000000u; };
-        tch::mma<S>(acc[n][0], a0[u].x, a1[u].x, a0[u].y, a1[u].y, x.x, x.y);
-        tch::mma<S>(acc[n][0], a0[u].z, a1[u].z, a0[u].w, a1[u].w, x.z, x.w);
-        tch::mma<S>(acc[n][1], a0[u].x, a1[u].x, a0[u].y, a1[u].y, turn(x.x), turn(x.y));
-        tch::mma<S>(acc[n][1], a0[u].z, a1[u].z, a0[u].w, a1[u].w, turn(x.z), turn(x.w));
-      }
-    if ((++count) * U >= RT_FLUSH || i0 + U * RT_WARPS >= groups) {
-      count = 0;
-#pragma unroll
-      for (int n = 0; n < NT; ++n)
-#pragma unroll
-        for (int h = 0; h < 2; ++h)
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            float s, e;
-            two_sum(hi[n][h][i], acc[n][h][i], s, e);
-            hi[n][h][i] = s;
-            lo[n][h][i] = __fadd_rn(lo[n][h][i], e);
-            acc[n][h][i] = 0.f;
-          }
-    }
-  }
-#pragma unroll
-  for (int n = 0; n < NT; ++n) {
-    __syncthreads();
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-      part[w][g + 8 * (i / 2)][2 * t + (i & 1)] = make_double2(widen(hi[n][0][i]) + widen(lo[n][0][i]),
-                                                               widen(hi[n][1][i]) + widen(lo[n][1][i]));
-    __syncthreads();
-    const int k = threadIdx.x / 8, r = threadIdx.x % 8;
-    if (k < 16 && k0 + k < nvec && 8 * n + r < R) {
-      double re = 0, im = 0;
-#pragma unroll
-      for (int q = 0; q < RT_WARPS; ++q) {
-        re += part[q][k][r].x;
-        im += part[q][k][r].y;
-      }
-      out[(b * nvec + k0 + k) * R + 8 * n + r] = make_float2((float)re, (float)im);
-    }
-  }
-}
-
 // c[a][k][r] = <phi_k^a, v_r> for R fields v
 void restrict_multi(Ctx& c, const Subspace& s, const uint4* v, int vprec, int R, void* cvec, int cprec) {
   const size_t ps = s.vec_bytes(c) / 16, vs = c.field_bytes(vprec) / 16;
@@ -687,17 +598,6 @@ void restrict_multi(Ctx& c, const Subspace& s, const uint4* v, int vprec, int R,
   HDCG_REQUIRE(R >= 1 && R <= RMAX, HDCG_ERR_ARG, "1..16 right-hand sides");
   const BlockArgs ba = block_args(c, s);
   ++c.launches;
-  if (s.prec == HDCG_F16 && vprec == HDCG_F16) {
-    const dim3 grid((unsigned)s.Vc, (unsigned)((s.nvec + 15) / 16));
-    if (R <= 8)
-      k_restrict_tc<f16_t, 1><<<grid, 32 * RT_WARPS, 0, c.stream>>>(s.vecs.as<uint4>(), ps, s.nvec, v, vs, R, ba,
-                                                                    (float2*)cvec);
-    else
-      k_restrict_tc<f16_t, 2><<<grid, 32 * RT_WARPS, 0, c.stream>>>(s.vecs.as<uint4>(), ps, s.nvec, v, vs, R, ba,
-                                                                    (float2*)cvec);
-    HDCG_CUDA(cudaGetLastError());
-    return;
-  }
   DISPATCH_SUB(s.prec, Sp, {
     DISPATCH_PREC(vprec, Sv, {
       using Rc = typename std::conditional<std::is_same<Sp, f64_t>::value, double, float>::type;

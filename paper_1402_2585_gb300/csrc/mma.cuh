@@ -1,5 +1,4 @@
-// The 16-bit warp-level matrix instruction of the hop passes (hop_tc.cuh) and the
-// restriction (coarse.cu).
+// The 16-bit warp-level matrix instruction of the hop passes (hop_tc.cuh).
 #pragma once
 
 #include <type_traits>
