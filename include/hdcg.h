@@ -458,6 +458,11 @@ int hdcg_get_phase_profile(hdcg_t h, double ms[6]);
  * keeps the faster; 1 or 2 forces one.  Both run the same MMAs in the same
  * order, so the results are identical.  HDCG_ERR_ARG outside 0..2. */
 int hdcg_set_coarse_tc_shape(hdcg_t h, int ctas_per_sm);
+/* Limit of a single wait inside the tensor-core stencil's pipeline (2 s by
+ * default): a call whose wait lasts longer returns HDCG_ERR_TIMEOUT, and the
+ * handle stays usable.  0 gives up at the first wait that is not over at once.
+ * HDCG_ERR_ARG outside 0..3600. */
+int hdcg_set_coarse_tc_wait(hdcg_t h, double seconds);
 
 /* Measurement: the mean device time (microseconds, CUDA events on the
  * handle's stream) of one tensor-core little Dirac stencil apply (k_capply_tc,

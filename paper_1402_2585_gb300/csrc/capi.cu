@@ -618,6 +618,14 @@ int hdcg_set_coarse_tc_shape(hdcg_t h, int ctas_per_sm) {
   return HDCG_OK;
 }
 
+int hdcg_set_coarse_tc_wait(hdcg_t h, double seconds) {
+  HDCG_ENTRY(h, {
+    HDCG_REQUIRE(seconds >= 0 && seconds <= 3600, HDCG_ERR_ARG, "the wait limit must be 0..3600 s");
+    c.tc_wait_ns = (uint64_t)(seconds * 1e9);
+  });
+  return HDCG_OK;
+}
+
 int hdcg_time_coarse_apply(hdcg_t h, int nrhs, int reps, double* us_per_apply) {
   HDCG_ENTRY(h, {
     check_ptr(us_per_apply, "us_per_apply");

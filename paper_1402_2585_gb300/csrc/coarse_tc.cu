@@ -317,6 +317,7 @@ struct TcArgs {
   // enough pairs to fill the chip.
   int nsplit;
   size_t part;
+  uint64_t wait_ns;    // limit of a wait for another role; waits for what was issued have WAIT_LIMIT_NS
 };
 __device__ __forceinline__ int split_begin(int s, int nsplit) { return s * 81 / nsplit; }
 
@@ -386,26 +387,28 @@ __global__ void __launch_bounds__(TC_THREADS, 2) k_capply_tc(TcArgs g, Reduction
       __syncwarp();
       const char* src = reinterpret_cast<const char*>(g.Atc) + ((size_t)pair * 81 + l0) * astep + (size_t)lane * g.a_gbytes;
       const int* nb = snb + (lane >= nA && lane < ncopy ? (lane - nA) * 81 : 0);
-      if (lane < ncopy) {
-        for (int l = l0; l < l1; ++l, ++it) {
-          if (!tc::mbar_wait(TC_EMPTY(s), ph ^ 1u)) {
-            ok = false;
-            atomicOr(g.err, 1u);
-            break;
-          }
-          if (lane == 0) tc::mbar_arrive_expect_tx(TC_FULL(s), g.copy_bytes);
-          // stage: [part 0: site 0, site 1][part 1: site 0, site 1][B site 0][B site 1]
+      for (int l = l0; l < l1; ++l, ++it) {
+        // All lanes issue or none: a stage that only some of them saw empty in time would
+        // get a part of its copies, which FULL and the wait before the exit do not cover.
+        const bool empty = lane >= ncopy || tc::mbar_wait(TC_EMPTY(s), ph ^ 1u, g.wait_ns);
+        ok = __all_sync(FULL_MASK, empty);
+        if (!ok) {
+          if (lane == 0) atomicOr(g.err, 1u);
+          break;
+        }
+        if (lane == 0) tc::mbar_arrive_expect_tx(TC_FULL(s), g.copy_bytes);
+        // stage: [part 0: site 0, site 1][part 1: site 0, site 1][B site 0][B site 1]
+        if (lane < ncopy)
           tc::bulk_g2s(ring + s * stage_bytes + doff,
                        lane < nA ? src : reinterpret_cast<const char*>(g.xtc) + (size_t)nb[l] * g.b_bytes, bytes,
                        TC_FULL(s));
-          src += astep;
-          if (++s == (uint32_t)g.stages) {
-            s = 0;
-            ph ^= 1u;
-          }
+        src += astep;
+        if (++s == (uint32_t)g.stages) {
+          s = 0;
+          ph ^= 1u;
         }
       }
-      ok = __all_sync(FULL_MASK, ok);   // every lane is done with snb before the next pair overwrites it
+      __syncwarp();   // every lane is done with snb before the next pair overwrites it
     }
     if (lane == 0) {
       // every copy issued has to land before the CTA exits
@@ -424,14 +427,14 @@ __global__ void __launch_bounds__(TC_THREADS, 2) k_capply_tc(TcArgs g, Reduction
       const uint32_t pstep = g.sites * g.a_sbytes;
       for (int p = blockIdx.x; ok && p < items; p += gridDim.x, ++np) {
         const int l0 = split_begin(p % g.nsplit, g.nsplit), l1 = split_begin(p % g.nsplit + 1, g.nsplit);
-        if (np > 0 && !tc::mbar_wait(ACC_EMPTY, (uint32_t)(np - 1) & 1u)) {
+        if (np > 0 && !tc::mbar_wait(ACC_EMPTY, (uint32_t)(np - 1) & 1u, g.wait_ns)) {
           ok = false;
           atomicOr(g.err, 4u);
           break;
         }
         tc::fence_after_sync();
         for (int l = l0; l < l1; ++l) {
-          if (!tc::mbar_wait(TC_FULL(s), ph)) {
+          if (!tc::mbar_wait(TC_FULL(s), ph, g.wait_ns)) {
             ok = false;
             atomicOr(g.err, 8u);
             break;
@@ -472,7 +475,7 @@ __global__ void __launch_bounds__(TC_THREADS, 2) k_capply_tc(TcArgs g, Reduction
     for (int r = 0; r < RMAX; ++r) inv[r] = r < g.R ? pow2f(-scale_exp(g.xmax[r])) : 0.f;
     int np = 0;
     for (int p = blockIdx.x; p < items; p += gridDim.x, ++np) {
-      const bool ok = tc::mbar_wait(ACC_FULL, (uint32_t)np & 1u);
+      const bool ok = tc::mbar_wait(ACC_FULL, (uint32_t)np & 1u, g.wait_ns);
       if (!__all_sync(FULL_MASK, ok)) {
         if (lane == 0) atomicOr(g.err, 32u);
         break;
@@ -624,6 +627,7 @@ static void launch_tc(Ctx& c, Coarse& A, int R, const float2* x, float2* y, cons
   a.parts = g.parts;
   a.nsplit = nsplit;
   a.part = A.Vc * A.nvec * (size_t)R;
+  a.wait_ns = c.tc_wait_ns;
   a.sexp = A.sexp.as<int>();
   const size_t smem = (size_t)g.stages * g.stage_bytes + (2 * g.stages + 3) * 8 + 16;
   static size_t smem_set = 0;

@@ -157,6 +157,7 @@ struct Ctx {
   DevMem scratch_f[NPREC][24]; // work fields per precision (slot roles: solver.cu; 20-23: hop autotuner)
   std::map<int, int> hop_tuned;  // (prec, pass, fused, reduction) -> chosen hop variant
   int hop_force = -1;            // >= 0: every hop launch uses this variant (hdcg_set_hop_variant)
+  uint64_t tc_wait_ns = 2000000000ull;   // limit of a wait in the tensor-core stencil's pipeline
   int tc_force = 0;              // 1, 2: the tensor-core stencil's CTAs per SM (hdcg_set_coarse_tc_shape)
   DevMem red_partials, red_ticket, scalars;
   PinnedMem pinned;              // scalars at 0, a solver's control block at 4096, error flags at 8064
@@ -277,6 +278,7 @@ void run_captured(Ctx& c, CapturedGraph& g, const std::vector<uintptr_t>& key_in
   }
   std::vector<uintptr_t> key = key_in;
   key.push_back((uintptr_t)alloc_epoch());
+  key.push_back((uintptr_t)c.tc_wait_ns);   // an argument of the captured stencil launches
   if (!g.exec || g.key != key) {
     g.reset();
     const long long l0 = c.launches;
