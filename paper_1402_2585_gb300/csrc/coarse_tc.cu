@@ -1084,7 +1084,7 @@ int coarse_cg_tc(Ctx& c, Coarse& A, int R, const void* rhs, void* sol, double to
   const std::vector<uintptr_t> key = {(uintptr_t)A.work.p, (uintptr_t)A.ctl.p, (uintptr_t)sol, (uintptr_t)A.Atc.p,
                                       (uintptr_t)A.xtc.p, (uintptr_t)A.tcs.p, (uintptr_t)c.red_partials.p,
                                       (uintptr_t)c.red_ticket.p, (uintptr_t)R, (uintptr_t)maxiter,
-                                      (uintptr_t)shift_bits};
+                                      (uintptr_t)shift_bits, (uintptr_t)nsplit};
   int queued = 0;
   int batch = std::max(2, A.last_iters);
   CCtlT& h = *c.pinned.at<CCtlT>(4096);

@@ -278,7 +278,9 @@ void run_captured(Ctx& c, CapturedGraph& g, const std::vector<uintptr_t>& key_in
   }
   std::vector<uintptr_t> key = key_in;
   key.push_back((uintptr_t)alloc_epoch());
-  key.push_back((uintptr_t)c.tc_wait_ns);   // an argument of the captured stencil launches
+  // an argument and the launch shape of the captured stencil launches
+  key.push_back((uintptr_t)c.tc_wait_ns);
+  key.push_back((uintptr_t)c.tc_force);
   if (!g.exec || g.key != key) {
     g.reset();
     const long long l0 = c.launches;
