@@ -288,7 +288,9 @@ int hdcg_coarse_apply_multi(hdcg_t h, const void* x, void* y, int nrhs);
  * lockstep iteration count.  HDCG_ERR_BREAKDOWN if the level-2 A-DEF2 solve
  * met (p, A p) <= 0 or a non-finite residual before the tolerance (inside
  * hdcg_solve the preconditioner keeps that right-hand side's last iterate
- * instead).  Synchronous. */
+ * instead).  The order of FP64 partial sums, and with it the last bits of a
+ * right-hand side, may depend on nrhs (small grids share one cluster launch
+ * while all right-hand sides fit it).  Synchronous. */
 int hdcg_coarse_solve(hdcg_t h, const void* b, void* x, int nrhs, double tol, int maxiter, int* iterations);
 
 /* y = A x exactly like hdcg_coarse_apply, but without allocating any device

@@ -264,10 +264,11 @@ static int hop_variant(Ctx& c, int prec, int pass, bool mob, const HopArgs& a, d
 
 // Threads per CTA.  FP64 and double-float kernels are built for 64.  The others
 // run 256, and 64 while that leaves SMs idle (152 SMs; an 8^4 x 8 field is 64
-// CTAs of 256 threads).
-static int hop_threads(const Ctx& c, int prec, int nrhs) {
+// CTAs of 256 threads).  The field decides, not the number of right-hand sides: the
+// CTAs' partial sums would otherwise be added in another order in a larger batch.
+static int hop_threads(const Ctx& c, int prec) {
   if (prec == HDCG_F64 || prec == HDCG_DF64) return 64;
-  return c.n5 * (size_t)nrhs < (size_t)152 * 256 * 2 ? 64 : 256;
+  return c.n5 < (size_t)152 * 256 * 2 ? 64 : 256;
 }
 
 // 16-bit storage with Ls >= 8 runs on the tensor cores unless a variant is
@@ -330,7 +331,7 @@ void launch_hop(Ctx& c, int pass, int prec, const uint4* in, const uint4* in2, u
   a.fstride = epi.nrhs > 1 ? epi.fstride : 0;
   a.al_mask = epi.mask;
   const bool tc = hop_use_tc(c, prec);
-  const int threads = hop_threads(c, prec, epi.nrhs);
+  const int threads = hop_threads(c, prec);
   const unsigned grid = tc ? hop_tc_grid(c) : (unsigned)((c.n5 + threads - 1) / threads);
   HDCG_REQUIRE(epi.nrhs >= 1 && epi.nrhs <= RMAX, HDCG_ERR_ARG, "1 <= right-hand sides <= 16");
   a.do_red = red_result != nullptr;
