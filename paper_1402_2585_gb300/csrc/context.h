@@ -155,7 +155,7 @@ struct Ctx {
   DevMem nbr[2];          // int32 [n4][8]: neighbour cb index of output site x (parity p)
   DevMem links[5][2];     // per link slot (F64, F32, F16, BF16) and output parity
   DevMem scratch_f[NPREC][24]; // work fields per precision (slot roles: solver.cu; 20-23: hop autotuner)
-  std::map<int, int> hop_tuned;  // (prec, pass, fused, reduction) -> chosen hop variant
+  std::map<int, int> hop_tuned;  // (prec, pass, fused, reduction, Moebius) -> chosen hop variant
   int hop_force = -1;            // >= 0: every hop launch uses this variant (hdcg_set_hop_variant)
   uint64_t tc_wait_ns = 2000000000ull;   // limit of a wait in the tensor-core stencil's pipeline
   int tc_force = 0;              // 1, 2: the tensor-core stencil's CTAs per SM (hdcg_set_coarse_tc_shape)

@@ -192,11 +192,11 @@ static void dispatch_hop(int prec, int v, int pass, bool mob, const HopArgs& a, 
   }
 }
 
-// Hop autotuner: the first launch of a (precision, pass, fused-CG) combination
-// times every register-budget variant on scratch fields (never on the
+// Hop autotuner: the first launch of a (precision, pass, fused-CG, reduction,
+// action) combination times every register-budget variant on scratch fields (never on the
 // caller's data, so in-place CG updates are not repeated) and keeps the fastest.
 static int hop_variant(Ctx& c, int prec, int pass, bool mob, const HopArgs& a, dim3 grid, int threads) {
-  const int key = ((prec * 4 + pass) * 2 + (a.cg_r ? 1 : 0)) * 2 + (a.do_red ? 1 : 0);
+  const int key = (((prec * 4 + pass) * 2 + (a.cg_r ? 1 : 0)) * 2 + (a.do_red ? 1 : 0)) * 2 + (mob ? 1 : 0);
   if (c.hop_force >= 0) {
     // a forced variant (hdcg_set_hop_variant); the packed variants exist for
     // FP32 and 16-bit storage only
@@ -236,8 +236,10 @@ static int hop_variant(Ctx& c, int prec, int pass, bool mob, const HopArgs& a, d
   // variants 0-3 only: the packed variants (4, 5) round differently, and a
   // timing-dependent pick among them would make two handles' results differ
   // in the last bits; they are slower on every measured lattice anyway and
-  // run only when forced
-  const int nv = 4;
+  // run only when forced.  So does variant 3 of FP64 storage, double-float
+  // arithmetic (H on 16^4 x 16: 6.1 ms against 3.7 for 0-2; 0.36 against 0.15 on
+  // 4^4 x 4; slower at every size between and beyond).
+  const int nv = prec == HDCG_F64 ? 3 : 4;
   for (int v = 0; v < nv; ++v) {
     dispatch_hop(prec, v, pass, mob, t, grid, threads, c.stream);  // warm-up
     HDCG_CUDA(cudaEventRecord(e0, c.stream));
