@@ -51,16 +51,6 @@ constexpr int TC_RPMAX = RMAX;                 // right-hand sides per launch
 constexpr uint32_t TC_RING_BYTES = 96 * 1024;  // two CTAs per SM
 constexpr uint32_t TC_RING_BYTES_1 = 192 * 1024;  // one CTA per SM
 
-int device_sms() {
-  static int n = 0;
-  if (!n) {
-    int dev = 0;
-    HDCG_CUDA(cudaGetDevice(&dev));
-    HDCG_CUDA(cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev));
-  }
-  return n;
-}
-
 void set_smem(const void* fn, size_t bytes) {
   HDCG_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
 }

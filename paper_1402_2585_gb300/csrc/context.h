@@ -80,6 +80,17 @@ struct DevMem {
   template <typename T> T* as() const { return reinterpret_cast<T*>(p); }
 };
 
+// SMs of the device that the process runs on
+inline int device_sms() {
+  static const int n = [] {
+    int dev = 0, sms = 0;
+    HDCG_CUDA(cudaGetDevice(&dev));
+    HDCG_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    return sms;
+  }();
+  return n;
+}
+
 // page-locked host memory for the scalars and control blocks that a solver loop
 // reads back: copies into it are queued and waited for once (a copy into pageable
 // memory waits for the stream by itself, every one of them)

@@ -265,12 +265,13 @@ static int hop_variant(Ctx& c, int prec, int pass, bool mob, const HopArgs& a, d
 }
 
 // Threads per CTA.  FP64 and double-float kernels are built for 64.  The others
-// run 256, and 64 while that leaves SMs idle (152 SMs; an 8^4 x 8 field is 64
-// CTAs of 256 threads).  The field decides, not the number of right-hand sides: the
-// CTAs' partial sums would otherwise be added in another order in a larger batch.
+// run 256, and 64 while that leaves SMs idle (fewer than two CTAs each; an 8^4 x 8
+// field is 64 CTAs of 256 threads on 152 SMs).  The field decides, not the number
+// of right-hand sides: the CTAs' partial sums would otherwise be added in another
+// order in a larger batch.
 static int hop_threads(const Ctx& c, int prec) {
   if (prec == HDCG_F64 || prec == HDCG_DF64) return 64;
-  return c.n5 < (size_t)152 * 256 * 2 ? 64 : 256;
+  return c.n5 < (size_t)device_sms() * 256 * 2 ? 64 : 256;
 }
 
 // 16-bit storage with Ls >= 8 runs on the tensor cores unless a variant is
@@ -281,10 +282,11 @@ static bool hop_use_tc(const Ctx& c, int prec) {
   return is_16bit(prec) && c.hop_force < 0 && c.Ls >= 8;
 }
 
-// persistent: as many CTAs as are resident, each warp striding over the sites
+// persistent: as many CTAs per right-hand side as are resident, each warp striding
+// over the sites (for one right-hand side and for several alike: the sums' order)
 static unsigned hop_tc_grid(const Ctx& c) {
   const size_t ctas = (c.n4 + tch::TC_WARPS - 1) / tch::TC_WARPS;
-  return (unsigned)std::min<size_t>(ctas, 152 * tch::tc_ctas(c.Ls / 8));
+  return (unsigned)std::min<size_t>(ctas, (size_t)device_sms() * tch::tc_ctas(c.Ls / 8));
 }
 
 void launch_hop(Ctx& c, int pass, int prec, const uint4* in, const uint4* in2, uint4* out,
