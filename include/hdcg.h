@@ -480,7 +480,7 @@ int hdcg_time_coarse_apply(hdcg_t h, int nrhs, int reps, double* us_per_apply);
  * shared memory (FP32 and 16-bit storage; measured slower than 0-3, and
  * rounding differently, so only run when forced).  By default (variant -1)
  * 16-bit storage with Ls >= 8 runs on the tensor cores (exact products of the
- * stored links and fields, FP32 sums); otherwise the first launch of each pass
+ * stored links and fields, FP32 sums truncated towards zero); otherwise the first launch of each pass
  * times variants 0-3 (0-2 for FP64 storage) and keeps the fastest
  * (0-2 and the 16-bit variant 3 give identical bits; for FP64 storage
  * variant 3's double-float arithmetic agrees with FP64 to about 1e-14); 0..5

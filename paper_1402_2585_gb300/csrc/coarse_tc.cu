@@ -836,7 +836,8 @@ __global__ void k_cgt_check(CCtlT* ctl, int R, int par, int maxiter) {
 // as four launches of 16 to 24 CTAs they took 33 us of an iteration, k_cgt_update
 // 18 of them.  One cluster of eight CTAs meets at two cluster barriers instead:
 // 14.8 us, with the scalars computed by one thread of a CTA.
-// With the split couplings (78 us a product on 128 of 152 SMs before, for 95 MB)
+// With the split couplings (78 us a product on 128 of 152 SMs before, for 170 MB:
+// the 95 MB of the operator, its 48 x 24 blocks padded to 64 x 32)
 // the batched solve of four sources on 16^4 x 16 went from 217 to 202 ms.
 // A thread owns the same (site, eight coefficients, right-hand side) items in every
 // phase.  |r|^2 in FP64, squares and sums: entries of FP32's whole range.

@@ -114,7 +114,7 @@ __device__ __forceinline__ dfl& operator*=(dfl& a, dfl b) { return a = a * b; }
 // renormalisation: e left to grow over more terms loses accuracy (on random
 // operands six products and the sum over eight hops: 3.3e-15 with double-float
 // products and sums, 4.2e-15 and more with one long compensated chain, 3.3e-15
-// with dot6 below and the hops summed in pairs).
+// with dot2 and sum3 below and the hops summed in pairs).
 __device__ __forceinline__ void dot_first(float& s, float& e, dfl a, dfl b) {
   s = __fmul_rn(a.hi, b.hi);
   e = __fmaf_rn(a.hi, b.hi, -s);

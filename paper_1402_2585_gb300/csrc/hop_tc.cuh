@@ -5,10 +5,12 @@
 // reals and out over the site's 24 reals, M built from the eight links and the
 // spin projectors.  The entries of (1 -+ gamma_mu) are 0, +-1 and +-i, so M holds
 // link components with a sign or with real and imaginary part exchanged: the
-// 16-bit links and the 16-bit fields enter mma.m16n8k16 exactly as stored, every
-// product is exact and the sums are FP32, as in the scalar pass.  (The scalar
-// pass projects first and rounds u -+ A l to FP32; here nothing is rounded
-// before the sum.)  M differs from site to site and is 24 columns wide, which
+// 16-bit links and the 16-bit fields enter mma.m16n8k16 exactly as stored and every
+// product is exact.  The FP32 sums are truncated towards zero (mma.cuh) where the
+// scalar pass rounds u -+ A l and its sums to nearest: against 64 bits both are as
+// far off as the 16-bit storage makes them (H of FP16 fields 3.16e-4 Shamir, 3.46e-4
+// Moebius, BF16 2.53e-3 and 2.77e-3, either pass within 0.1 %), and <psi, H psi> moves by
+// 1e-7 of itself on average, towards zero.  M differs from site to site and is 24 columns wide, which
 // rules out tcgen05: its M = 128 rows would share one shared-memory operand.
 //
 // Shape: m16 are 16 slices of one 4D site (Ls 32: two tiles, Ls 8: half a tile),

@@ -10,7 +10,9 @@ namespace tch {
 
 // d += a b, m16n8k16: fragment rows g, g + 8 (g = lane / 4), k 2 t, 2 t + 1 and
 // 2 t + 8, 2 t + 9 (t = lane % 4), column g of b, columns 2 t, 2 t + 1 of d; exact
-// 16-bit products, FP32 sums
+// 16-bit products.  The FP32 sum is truncated towards zero: to 1 it adds nothing of
+// 3/4 ulp and 1 of 7/4 ulp, measured.  Long sums of one sign drift (512 products
+// summed in one accumulator: 2.6e-6), so contractions with few terms only.
 template <typename St>
 __device__ __forceinline__ void mma(float (&d)[4], unsigned a0, unsigned a1, unsigned a2, unsigned a3, unsigned b0,
                                     unsigned b1) {
