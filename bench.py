@@ -2,7 +2,10 @@
 with the fine Mpc^dag Mpc hop kernels' achieved bandwidth against the HBM roofline.
 
 One step = one full HDCG solve of H x = b to a true FP64 residual of ``tol``
-(a Gaussian source; ``--nrhs`` of them together), inputs resident in HBM.  The
+(a Gaussian source; ``--nrhs`` of them together), inputs resident in HBM.  Step k
+solves the workload's source moved by k * SOURCE_STEP sites, as do the end-to-end
+steps: the outer iterations of one source move by factors with rounding (61 to
+470 over eight sources), so a single source says little about the solver.  The
 default workload is the physical-point-like lattice: 32^3 x 64, Ls 16 Moebius
 (b 1.5, c 0.5), M5 1.8, m 0.001, links exp(i 0.45 H); three levels (4^4
 blocks with Nvec 40, then 2^4 blocks of the coarse lattice with Nvec 24);
@@ -50,20 +53,25 @@ PREC = {"f64": 0, "f32": 1, "f16": 2, "bf16": 3}
 
 # Fine H applies (outer + preconditioner + FP64 residual) per right-hand side
 # of one HDCG solve, from the GPU arm's solve statistics on each workload (a
-# property of the algorithm on that input).  The reference arm, which runs no
+# property of the algorithm on that input).  The default's is that of a solve in 91
+# iterations: with an FP32 preconditioner two sources took 67 and 106, with the FP16
+# one 20 sources took 57 to 470, and the oracle rounds neither.  The reference arm, which runs no
 # GPU code, scales the oracle's per-apply time by it; the GPU arm reports its
 # measured count beside this figure (``h_applies_per_rhs``).
 H_APPLIES_PER_RHS = {DEFAULT_WORKLOAD: 824, "cfg2_16x16x16x16_ls16_shamir": 140}
 
-# DRAM bytes (read + write) per hop_kernel launch of the outer precision from
+# DRAM bytes (read + write) per launch of the sloppy precision's hop passes from
 # one ncu capture of the current kernel, per workload; None once the kernel
 # changes (the counters then no longer describe it).
 HOP_TRAFFIC = {
-    # ncu (dram__bytes_read.sum + dram__bytes_write.sum) of the four FP16 passes
-    # of one H at this size (bench.py --apply-only 3, no fused CG epilogue),
-    # averaged per launch: 2.19, 3.32, 2.14 and 3.33 GB for passes A-D
-    DEFAULT_WORKLOAD: 2.745e9,
+    # scalar kernel: 2.745e9.  The tensor-core pass has been captured at 24^3 x 48
+    # only (cfg3, four passes of one H: 789 MB a launch, 1.08 of the algorithmic bytes)
+    DEFAULT_WORKLOAD: None,
 }
+
+
+SOURCE_STEP = 4099   # sites between the sources of consecutive steps (prime)
+E2E_STEPS = 5
 
 
 def hop_flops_per_site(w) -> int:
@@ -351,8 +359,8 @@ def run_ours(args, w):
     # pinned host copies (the end-to-end run copies them in and out every step)
     bp = torch.empty(bh.shape, dtype=torch.complex128, pin_memory=not args.no_e2e)
     bp.numpy()[...] = bh
-    del bh
-    b = bp.to(dev)
+    b0 = bp.to(dev)
+    b = b0.clone()
     x = torch.zeros_like(b)
     flush = torch.empty(512 * 1024 * 1024 // 4, dtype=torch.float32, device=dev)
 
@@ -371,7 +379,8 @@ def run_ours(args, w):
     launches0 = h.launch_count()
     times, stats = [], []
     torch.cuda.nvtx.range_push("timed")
-    for _ in range(args.steps):
+    for k in range(args.steps):
+        b.copy_(torch.roll(b0, k * SOURCE_STEP, dims=1))
         flush.zero_()
         e0 = torch.cuda.Event(enable_timing=True)
         e1 = torch.cuda.Event(enable_timing=True)
@@ -388,7 +397,10 @@ def run_ours(args, w):
     t_solve = max_over_ranks(statistics.mean(times), world, dev)
     s0 = stats[-1]
 
-    # profile pass: one more solve with event timing of every hop launch and phase
+    n_h = statistics.mean(s["n_mdagm_outer"] + s["n_mdagm_sloppy"] + s["n_mdagm_f64"] for s in stats)
+
+    # profile pass: one more solve (of the last step's source) with event timing of
+    # every hop launch and phase
     flush.zero_()
     torch.cuda.synchronize(dev)
     h.set_profiling(True)
@@ -403,8 +415,8 @@ def run_ours(args, w):
     h.set_profiling(False)
     coarse_rl = coarse_roofline(h, w, args)
 
-    # the solution's true residual, recomputed by the library's FP64-accurate operator
-    true_res = s0["true_residual"]
+    # the solutions' true residual, recomputed by the library's FP64-accurate operator
+    true_res = max(s["true_residual"] for s in stats)
 
 
     # plain red-black CG on the same GPU (FP32 with FP64 reliable updates), one
@@ -430,7 +442,7 @@ def run_ours(args, w):
     speedup = {"value": t_cg / t_hdcg_rhs if t_hdcg_rhs > 0 else None,
                "kind": "per right-hand side" + ("" if cg_conv else ", lower bound (CG not converged)"),
                "hdcg_seconds_per_rhs": t_hdcg_rhs}
-    del b, x
+    del b, b0, x
     torch.cuda.empty_cache()
 
     # the batch of spin-colour point sources (12 for the physical-point-like
@@ -475,7 +487,8 @@ def run_ours(args, w):
     if not args.no_e2e:
         xp = torch.zeros(bp.shape, dtype=bp.dtype, pin_memory=True)
         ts_e2e = []
-        for _ in range(1):
+        for k in range(min(args.steps, E2E_STEPS)):
+            bp.numpy()[...] = np.roll(bh, k * SOURCE_STEP, axis=1)
             flush.zero_()
             torch.cuda.synchronize(dev)
             t0 = time.perf_counter()
@@ -485,6 +498,7 @@ def run_ours(args, w):
         e2e = {"value": statistics.mean(ts_e2e), "unit": "s", "h2d_bytes_per_step": nbytes,
                "d2h_bytes_per_step": nbytes}
         del bp, xp
+    del bh
 
     if rank != 0:
         if world > 1:
@@ -493,7 +507,6 @@ def run_ours(args, w):
     peak, peak_kind = peaks()
     pname = {0: "f64", 1: "f32"}[outer]
     sloppy = {0: "f64", 1: "f32", 2: "f16", 3: "bf16"}[prec]
-    n_h = s0["n_mdagm_outer"] + s0["n_mdagm_sloppy"] + s0["n_mdagm_f64"]
     cpu = None
     if world == 1 and not args.no_cpu_baseline:
         per_site = oracle_h_seconds_per_site(w)
@@ -528,7 +541,8 @@ def run_ours(args, w):
         "clocks": clocks,
         "plain_cg": plain_cg,
         "speedup_vs_plain_cg": speedup,
-        "hdcg": {"iterations": s0["iterations"], "coarse_iterations": s0["coarse_iterations"],
+        "hdcg": {"iterations_per_step": [s["iterations"] for s in stats],
+                 "iterations": s0["iterations"], "coarse_iterations": s0["coarse_iterations"],
                  "coarse_iterations_max": s0["coarse_iterations_max"],
                  "n_mdagm_outer": s0["n_mdagm_outer"], "n_mdagm_sloppy": s0["n_mdagm_sloppy"],
                  "n_mdagm_f64": s0["n_mdagm_f64"], "reliable_updates": s0["reliable_updates"],
@@ -575,6 +589,11 @@ def coarse_roofline(h, w, args):
     return out
 
 
+def hop_kernel_name(w, pname):
+    """16-bit storage with Ls >= 8 runs on the tensor cores."""
+    return "hop_tc_kernel" if pname in ("f16", "bf16") and w.Ls >= 8 else "hop_kernel"
+
+
 def hop_flop_rate(w, hop_all, pname):
     """Flop rate of the roofline kernel's launches: every four launches are one
     H over the lattice's odd 5D sites (the bench's solves have one right-hand
@@ -584,11 +603,11 @@ def hop_flop_rate(w, hop_all, pname):
         return None
     flops = hp["launches"] / 4.0 * n5_of(w) * hop_flops_per_site(w)
     return {"flop_per_site_per_H": hop_flops_per_site(w), "achieved": flops / (hp["ms"] / 1e3) / 1e12,
-            "unit": "TFLOP/s", "kernel": f"hop_kernel ({pname} storage), the roofline kernel's launches"}
+            "unit": "TFLOP/s", "kernel": f"{hop_kernel_name(w, pname)} ({pname} storage), the roofline kernel's launches"}
 
 
 def roofline(w, hop_all, pname, peak, peak_kind, nrhs):
-    """The dominant kernel's roofline: hop_kernel passes in the sloppy storage
+    """The dominant kernel's roofline: the hop passes in the sloppy storage
     precision (most of the solve's fine-operator work).  achieved = algorithmic
     bytes per launch / mean launch time (CUDA events on the library's stream,
     profiled solve), in two accountings: the operator's own bytes ((240 +
@@ -605,7 +624,7 @@ def roofline(w, hop_all, pname, peak, peak_kind, nrhs):
             "traffic": HOP_TRAFFIC.get(w.name) if pname == "f16" else None,
             "traffic_note": ("ncu, unfused operator passes of one H at this size, mean per launch"
                              if HOP_TRAFFIC.get(w.name) and pname == "f16" else None),
-            "kernel": f"hop_kernel ({pname} storage, 4 passes per H)", "launches": hp["launches"],
+            "kernel": f"{hop_kernel_name(w, pname)} ({pname} storage, 4 passes per H)", "launches": hp["launches"],
             "avg_launch_us": per_launch_s * 1e6, "bytes_per_launch": b_fused,
             "achieved_operator_bytes_only": b_op / per_launch_s / 1e9,
             "frac_operator_bytes_only": b_op / per_launch_s / 1e9 / peak,

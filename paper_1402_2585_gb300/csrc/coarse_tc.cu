@@ -835,7 +835,8 @@ __global__ void k_cgt_check(CCtlT* ctl, int R, int par, int maxiter) {
 // the operand and the bookkeeping need each other's results over the whole grid:
 // as four launches of 16 to 24 CTAs they took 33 us of an iteration, k_cgt_update
 // 18 of them.  One cluster of eight CTAs meets at two cluster barriers instead:
-// 14.8 us, with the scalars computed by one thread of a CTA.
+// 14.8 us, with the scalars computed by one thread of a CTA; 18 with |r|^2 in FP64
+// (an iteration 62.5 -> 66 us for 4 right-hand sides, 93 -> 105 for 16).
 // With the split couplings (78 us a product on 128 of 152 SMs before, for 170 MB:
 // the 95 MB of the operator, its 48 x 24 blocks padded to 64 x 32)
 // the batched solve of four sources on 16^4 x 16 went from 217 to 202 ms.
